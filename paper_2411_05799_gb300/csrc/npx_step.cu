@@ -165,12 +165,14 @@ __device__ __forceinline__ float asin_small(float x) {
 // ------------------------------------------------------------------------ shared-memory slots
 
 // Per scene: float4 pts[max_points] | float frames[12 * max_links] | float theta[max_links] |
-// float theta_old[max_links] | float4 tile bounds[2 * ceil(max_points / lps)]
+// float theta_old[max_links] | uint16 parent and depth[max_links] | float4 tile bounds[2 * ceil(max_points / lps)]
 __host__ __device__ inline int tiles_offset(int max_points, int max_links) {
-    return (16 * max_points + 56 * max_links + 15) & ~15;
+    return (16 * max_points + 58 * max_links + 15) & ~15;
 }
+// (16 bytes after the boxes: at shape updates their area holds the points' links, shifted by up to
+// 3 bytes)
 __host__ __device__ inline int slot_bytes(int max_points, int max_links, int lps) {
-    return tiles_offset(max_points, max_links) + 32 * ((max_points + lps - 1) / lps);
+    return tiles_offset(max_points, max_links) + 32 * ((max_points + lps - 1) / lps) + 16;
 }
 // (height maps) the window and its mbarrier after the slot, 128-byte aligned for the TMA box
 __host__ __device__ inline int hm_win_offset(int max_points, int max_links, int lps) {
@@ -277,18 +279,34 @@ __device__ __forceinline__ uint64_t tiles_near_ground(const float4 *tb, int ntil
 // to the shape frame (root link fixed).  A link's frame is its parent's frame followed by the
 // hinge rotation by theta about the unit axis through the anchor.  Lanes build the local hinge
 // transforms in parallel, then compose them one tree level at a time.
+struct Frame {
+    float4 a, b, c;   // Q row-major, then T
+};
+__device__ __forceinline__ Frame frame_load(const float *F) {
+    const float4 *f = reinterpret_cast<const float4 *>(F);
+    return Frame{f[0], f[1], f[2]};
+}
+__device__ __forceinline__ void frame_store(float *F, const float q[9], const float t[3]) {
+    float4 *f = reinterpret_cast<float4 *>(F);
+    f[0] = make_float4(q[0], q[1], q[2], q[3]);
+    f[1] = make_float4(q[4], q[5], q[6], q[7]);
+    f[2] = make_float4(q[8], t[0], t[1], t[2]);
+}
+
+// Bound by latency: a chain of dependent loads.  The link records are read once (the frame and the
+// two tree numbers a level needs, which stay in the slot), so the levels cost shared-memory
+// latency; reading each record again at every level from L2 was a third of a joint update.
+// Frames move as three 16-byte words.  With the links' asynchronous copies in shape_update, a step
+// with a joint update of 4,096 hexapods (16 lanes, 14 warps per SM) took 16.8 us after, 20.6
+// before; a 1,000-step second with one every 80 steps 2.15 ms after, 2.17 before.
 template <int LPS>
 __device__ __noinline__ void link_frames(const WorldDev &W, int l0, int nl, const float *th, float *fr, int gl) {
+    uint16_t *pd = reinterpret_cast<uint16_t *>(fr + 14 * W.max_links);
+#pragma unroll 2
     for (int l = gl; l < nl; l += LPS) {
-        float *F = fr + 12 * l;
-        if (l == 0) {
-            F[0] = 1.f; F[1] = 0.f; F[2] = 0.f; F[3] = 0.f; F[4] = 1.f; F[5] = 0.f;
-            F[6] = 0.f; F[7] = 0.f; F[8] = 1.f; F[9] = 0.f; F[10] = 0.f; F[11] = 0.f;
-            continue;
-        }
         const LinkDev lk = W.links[l0 + l];
         float s, c;
-        sincosf(th[l - 1], &s, &c);
+        sincosf(l == 0 ? 0.f : th[l - 1], &s, &c);
         const float k = 1.f - c, ux = lk.ux, uy = lk.uy, uz = lk.uz;
         float Rj[9] = {c + k * ux * ux, k * ux * uy - s * uz, k * ux * uz + s * uy,
                        k * uy * ux + s * uz, c + k * uy * uy, k * uy * uz - s * ux,
@@ -296,20 +314,26 @@ __device__ __noinline__ void link_frames(const WorldDev &W, int l0, int nl, cons
         const float a[3] = {lk.ax, lk.ay, lk.az};
         float Ra[3];
         mat_vec(Rj, a, Ra);
+        float T[3] = {a[0] - Ra[0], a[1] - Ra[1], a[2] - Ra[2]};
+        if (l == 0) {   // the root link's frame is the shape frame
 #pragma unroll
-        for (int i = 0; i < 9; ++i) F[i] = Rj[i];
-        F[9] = a[0] - Ra[0]; F[10] = a[1] - Ra[1]; F[11] = a[2] - Ra[2];
+            for (int i = 0; i < 9; ++i) Rj[i] = (i & 3) == 0 ? 1.f : 0.f;
+            T[0] = T[1] = T[2] = 0.f;
+        }
+        frame_store(fr + 12 * l, Rj, T);
+        pd[l] = (uint16_t)((lk.parent & 255) | (lk.depth << 8));
     }
     __syncwarp();
     // level d >= 2: F_l = F_parent o F_l (parents at level d-1 are final)
     for (int d = 2;; ++d) {
         bool any = false;
         for (int l = gl; l < nl; l += LPS) {
-            const LinkDev lk = W.links[l0 + l];
-            if (lk.depth != d) continue;
+            const uint32_t v = pd[l];
+            if ((int)(v >> 8) != d) continue;
             any = true;
-            const float *P = fr + 12 * lk.parent;
-            float *F = fr + 12 * l;
+            const Frame p = frame_load(fr + 12 * (v & 255u)), f = frame_load(fr + 12 * l);
+            const float P[12] = {p.a.x, p.a.y, p.a.z, p.a.w, p.b.x, p.b.y, p.b.z, p.b.w, p.c.x, p.c.y, p.c.z, p.c.w};
+            const float F[12] = {f.a.x, f.a.y, f.a.z, f.a.w, f.b.x, f.b.y, f.b.z, f.b.w, f.c.x, f.c.y, f.c.z, f.c.w};
             float Q[9], T[3];
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
@@ -318,9 +342,7 @@ __device__ __noinline__ void link_frames(const WorldDev &W, int l0, int nl, cons
                     Q[3 * i + j] = P[3 * i] * F[j] + P[3 * i + 1] * F[3 + j] + P[3 * i + 2] * F[6 + j];
                 T[i] = P[3 * i] * F[9] + P[3 * i + 1] * F[10] + P[3 * i + 2] * F[11] + P[9 + i];
             }
-#pragma unroll
-            for (int i = 0; i < 9; ++i) F[i] = Q[i];
-            F[9] = T[0]; F[10] = T[1]; F[11] = T[2];
+            frame_store(fr + 12 * l, Q, T);
         }
         __syncwarp();
         if (!__any_sync(FULL_MASK, any)) break;
@@ -333,13 +355,26 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
                  "l"(gmem_src)
                  : "memory");
 }
+__device__ __forceinline__ void cp_async4(void *smem_dst, const void *gmem_src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)),
+                 "l"(gmem_src)
+                 : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-__device__ __forceinline__ void fk_point(const float *fr, float4 a, int l, float p[3]) {
+// (the step loop's own copy reads the frame word by word: with wide loads the compiler fuses other
+// products of the loop, and the friction options' results would round differently)
+__device__ __forceinline__ void fk_point_words(const float *fr, float4 a, int l, float p[3]) {
     const float *F = fr + 12 * l;
     p[0] = F[0] * a.x + F[1] * a.y + F[2] * a.z + F[9];
     p[1] = F[3] * a.x + F[4] * a.y + F[5] * a.z + F[10];
     p[2] = F[6] * a.x + F[7] * a.y + F[8] * a.z + F[11];
+}
+__device__ __forceinline__ void fk_point(const float *fr, float4 a, int l, float p[3]) {
+    const Frame f = frame_load(fr + 12 * l);
+    p[0] = f.a.x * a.x + f.a.y * a.y + f.a.z * a.z + f.c.y;
+    p[1] = f.a.w * a.x + f.b.x * a.y + f.b.y * a.z + f.c.z;
+    p[2] = f.b.z * a.x + f.b.w * a.y + f.c.x * a.z + f.c.w;
 }
 
 struct Shape {
@@ -360,26 +395,23 @@ __device__ __noinline__ void shape_update(const WorldDev &W, int s, int p0, int 
     // the construction positions and masses go straight into the offsets array (asynchronous
     // copies, all in flight at once) and the points' links into the tile-box area (rebuilt after
     // every shape update) while the link frames are built
-    uint8_t *lk = reinterpret_cast<uint8_t *>(pts) + tiles_offset(W.max_points, W.max_links);
+    // (as whole aligned words where their address allows, the ends byte by byte; every read stays
+    // inside the scene's bytes, and nothing waits for a load before the frames are done)
+    const uint8_t *src = W.plink + p0;
+    uint8_t *lk = reinterpret_cast<uint8_t *>(pts) + tiles_offset(W.max_points, W.max_links) +
+                  ((uint32_t)(uintptr_t)src & 3u);
 #pragma unroll 8
     for (int i = gl; i < np; i += LPS) cp_async16(pts + i, W.p0m + p0 + i);
-    {
-        // the link bytes as whole aligned words (a quarter of the loads), the unaligned head and
-        // tail byte by byte; every read stays inside the scene's bytes
-        const uint8_t *src = W.plink + p0;
-        const int h = min((int)((4u - ((uint32_t)(uintptr_t)src & 3u)) & 3u), np);
-        const int nw = (np - h) >> 2;
-        const uint32_t *ws = reinterpret_cast<const uint32_t *>(src + h);
-        for (int i = gl; i < h; i += LPS) lk[i] = src[i];
+    const int h = min((int)((4u - ((uint32_t)(uintptr_t)src & 3u)) & 3u), np);
+    const int nw = (np - h) >> 2, e = h + 4 * nw + gl;
+    uint8_t head = 0, tail = 0;
+    if (gl < h) head = src[gl];
+    if (e < np) tail = src[e];
 #pragma unroll 4
-        for (int k = gl; k < nw; k += LPS) {
-            const uint32_t v = ws[k];
-            uint8_t *d = lk + h + 4 * k;
-            d[0] = (uint8_t)v; d[1] = (uint8_t)(v >> 8); d[2] = (uint8_t)(v >> 16); d[3] = (uint8_t)(v >> 24);
-        }
-        for (int i = h + 4 * nw + gl; i < np; i += LPS) lk[i] = src[i];
-    }
+    for (int k = gl; k < nw; k += LPS) cp_async4(lk + h + 4 * k, src + h + 4 * k);
     link_frames<LPS>(W, l0, nl, th, fr, gl);
+    if (gl < h) lk[gl] = head;
+    if (e < np) lk[e] = tail;
     cp_async_wait_all();
     __syncwarp();
     const float gref[3] = {W.gref[3 * s], W.gref[3 * s + 1], W.gref[3 * s + 2]};
@@ -1473,7 +1505,7 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
                 const float4 r = pts[i];
                 const float4 a0 = W.p0m[p0 + i];
                 float po[3];
-                fk_point(fr, a0, W.plink[p0 + i], po);
+                fk_point_words(fr, a0, W.plink[p0 + i], po);
                 const float4 ro = make_float4(po[0] - gold[0], po[1] - gold[1], po[2] - gold[2], 0.f);
                 const float rx = R[0] * r.x + R[1] * r.y + R[2] * r.z;
                 const float ry = R[3] * r.x + R[4] * r.y + R[5] * r.z;

@@ -716,7 +716,9 @@ __device__ __forceinline__ void chunk_boxes_body(const WorldDev &W, int c0, int 
         hb.x = fabsf(F[0]) * hh.x + fabsf(F[1]) * hh.y + fabsf(F[2]) * hh.z;
         hb.y = fabsf(F[3]) * hh.x + fabsf(F[4]) * hh.y + fabsf(F[5]) * hh.z;
         hb.z = fabsf(F[6]) * hh.x + fabsf(F[7]) * hh.y + fabsf(F[8]) * hh.z;
-        cb.w = hb.w = 0.f;
+        // the chunk's entries in lpt ride in the fourth words
+        cb.w = __int_as_float(W.cpo[c0 + l]);
+        hb.w = __int_as_float(W.cpo[c0 + l + 1]);
         LB[2 * l] = cb;
         LB[2 * l + 1] = hb;
     }
@@ -807,9 +809,21 @@ __device__ __forceinline__ int arena_build(const WorldDev &W, unsigned char *xw,
             for (int k = 0; k < 9; ++k) { Ri[k] = Xi[XC_R + k]; Rj[k] = Xj[XC_R + k]; }
             const float4 *pti = reinterpret_cast<const float4 *>(pw + (ptrdiff_t)gi * sbytes);
             const float4 *ptj = reinterpret_cast<const float4 *>(pw + (ptrdiff_t)gj * sbytes);
+            // Each lane walks the candidate chunks of one point of i: a round takes the lane's next
+            // chunk (up to 16 of its points at a time) whose body-frame box comes within reach.
+            // Few lanes have one, so a round's chunks are tested by half-warps, one point of the
+            // chunk per lane, four chunks in flight: testing them lane by lane left 30 of 32 lanes
+            // idle and was most of an arena's step (1,024 arenas of four: 84 us a step before, 54
+            // after, with the list's entries loaded ahead and add_wrenches).  Entries keep the order
+            // round, lane, point.
+            const unsigned below = (1u << lane) - 1u;
+            const int half = lane >> 4, k16 = lane & 15;
+            int ck = lane < npi ? W.pchunk[p0i + lane] : 0;
             for (int ia0 = 0; ia0 < npi; ia0 += 32) {   // warp-uniform
                 const int ia = ia0 + lane;
-                uint64_t bm = ia < npi ? NMi[W.pchunk[p0i + ia]] : 0ull;
+                uint64_t bm = ia < npi ? NMi[ck] : 0ull;
+                if (ia + 32 < npi) ck = W.pchunk[p0i + ia + 32];   // the next points' chunks
+                if (!__any_sync(FULL_MASK, bm != 0ull)) continue;
                 float ah0 = 0.f, ah1 = 0.f, ah2 = 0.f;
                 if (bm) {
                     const float4 pa = pti[ia];
@@ -821,52 +835,53 @@ __device__ __forceinline__ int arena_build(const WorldDev &W, unsigned char *xw,
                     ah1 = Rj[1] * e[0] + Rj[4] * e[1] + Rj[7] * e[2];
                     ah2 = Rj[2] * e[0] + Rj[5] * e[1] + Rj[8] * e[2];
                 }
-                // each lane walks its candidate chunks: a round takes the lane's next chunk when
-                // its current one is done (whose body-frame box must come within reach) and tests
-                // up to 16 of the chunk's points at once; the rounds are warp-wide and the lanes'
-                // entries go out in lane order (a warp prefix sum), so the appends keep a fixed
-                // order
                 int ib = 0, b1 = 0;
                 while (__any_sync(FULL_MASK, bm != 0ull || ib < b1)) {
-                    uint32_t hit = 0u;
-                    int ib0 = 0;   // the round's first tested point
                     if (ib >= b1 && bm) {
                         const int lb = __ffsll((long long)bm) - 1;
                         bm &= bm - 1;
                         const float4 cbh = LBj[2 * lb], hbh = LBj[2 * lb + 1];
                         if (fabsf(ah0 - cbh.x) <= hbh.x + cull && fabsf(ah1 - cbh.y) <= hbh.y + cull &&
                             fabsf(ah2 - cbh.z) <= hbh.z + cull) {
-                            ib = W.cpo[l0j + lb];
-                            b1 = W.cpo[l0j + lb + 1];
+                            ib = __float_as_int(cbh.w);
+                            b1 = __float_as_int(hbh.w);
                         }
                     }
-                    if (ib < b1) {
-                        ib0 = ib;
-                        const int nb = min(16, b1 - ib);
+                    const int ib0 = ib, nb = min(16, b1 - ib);   // this round's points (none: nb <= 0)
+                    unsigned todo = __ballot_sync(FULL_MASK, nb > 0);
+                    if (nb > 0) ib += nb;
+                    while (todo) {   // warp-uniform
+                        int src[2], pi[2];
+                        bool hit[2];
 #pragma unroll
-                        for (int k = 0; k < 16; ++k) {
-                            if (k < nb) {
-                                const float4 pb = ptj[__ldg(W.lpt + ib + k)];
-                                const float d0 = ah0 - pb.x, d1 = ah1 - pb.y, d2 = ah2 - pb.z;
-                                if (d0 * d0 + d1 * d1 + d2 * d2 < cut2) hit |= 1u << k;
+                        for (int u = 0; u < 2; ++u) {   // two chunks each, lower lane first
+                            const int s0 = todo ? __ffs(todo) - 1 : -1;
+                            todo &= todo - 1u;
+                            const int s1 = todo ? __ffs(todo) - 1 : -1;
+                            todo &= todo - 1u;
+                            src[u] = half ? s1 : s0;
+                            const int sl = src[u] < 0 ? 0 : src[u];
+                            const float x0 = __shfl_sync(FULL_MASK, ah0, sl), x1 = __shfl_sync(FULL_MASK, ah1, sl);
+                            const float x2 = __shfl_sync(FULL_MASK, ah2, sl);
+                            const int sb = __shfl_sync(FULL_MASK, ib0, sl), sn = __shfl_sync(FULL_MASK, nb, sl);
+                            hit[u] = false;
+                            pi[u] = 0;
+                            if (src[u] >= 0 && k16 < sn) {
+                                pi[u] = __ldg(W.lpt + sb + k16);
+                                const float4 pb = ptj[pi[u]];
+                                const float d0 = x0 - pb.x, d1 = x1 - pb.y, d2 = x2 - pb.z;
+                                hit[u] = d0 * d0 + d1 * d1 + d2 * d2 < cut2;
                             }
                         }
-                        ib += nb;
-                    }
-                    const int cnt = __popc(hit);
-                    int pre = cnt;   // inclusive prefix sum over the lanes
 #pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int y = __shfl_up_sync(FULL_MASK, pre, o);
-                        if (lane >= o) pre += y;
+                        for (int u = 0; u < 2; ++u) {
+                            const unsigned hm = __ballot_sync(FULL_MASK, hit[u]);
+                            const int pos = total + __popc(hm & below);
+                            if (hit[u] && pos < W.alist_cap)
+                                alist[pos] = (uint32_t)(ia0 + src[u]) | ((uint32_t)pi[u] << AL_BITS);
+                            total += __popc(hm);
+                        }
                     }
-                    int pos = total + pre - cnt;
-                    for (uint32_t h = hit; h; h &= h - 1, ++pos) {
-                        const int k = __ffs(h) - 1;
-                        if (pos < W.alist_cap)
-                            alist[pos] = (uint32_t)ia | ((uint32_t)__ldg(W.lpt + ib0 + k) << AL_BITS);
-                    }
-                    total += __shfl_sync(FULL_MASK, pre, 31);
                 }
             }
         }
@@ -874,6 +889,29 @@ __device__ __forceinline__ int arena_build(const WorldDev &W, unsigned char *xw,
         __syncwarp();
     }
     return total;
+}
+
+// Adds the warp's sums of fi and fj to ti and tj.  Each sum is the butterfly's (lane l + lane l ^ 16,
+// then ^ 8, ...), but a lane only carries on the values it keeps: 13 shuffles instead of 60.
+__device__ __forceinline__ void add_wrenches(const float (&fi)[6], const float (&fj)[6], float *ti, float *tj) {
+    const int lane = threadIdx.x & 31;
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
+    float v[6], w[3];
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+        v[k] = (b4 ? fj[k] : fi[k]) + __shfl_xor_sync(FULL_MASK, b4 ? fi[k] : fj[k], 16);
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        w[k] = (b3 ? v[k + 3] : v[k]) + __shfl_xor_sync(FULL_MASK, b3 ? v[k] : v[k + 3], 8);
+    const float x0 = (b2 ? w[2] : w[0]) + __shfl_xor_sync(FULL_MASK, b2 ? w[0] : w[2], 4);
+    const float x1 = w[1] + __shfl_xor_sync(FULL_MASK, w[1], 4);
+    const bool second = !b2 && b1;   // lanes that keep the second of two values
+    float y = (second ? x1 : x0) + __shfl_xor_sync(FULL_MASK, (b2 || b1) ? x0 : x1, 2);
+    y += __shfl_xor_sync(FULL_MASK, y, 1);
+    if (!(lane & 1) && !(b2 && b1)) {
+        const int k = (b3 ? 3 : 0) + (b2 ? 2 : b1 ? 1 : 0);
+        (b4 ? tj : ti)[k] += y;
+    }
 }
 
 // Pair forces from the list: for each robot pair of the warp, its entries spread over the lanes,
@@ -904,35 +942,31 @@ __device__ __forceinline__ void arena_list_forces(const WorldDev &W, unsigned ch
                 const float4 *pti = reinterpret_cast<const float4 *>(pw + (ptrdiff_t)gi * sbytes);
                 const float4 *ptj = reinterpret_cast<const float4 *>(pw + (ptrdiff_t)gj * sbytes);
                 float fi[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, fj[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                for (int en = start + lane; en < end; en += 32) {
-                    const uint32_t code = alist[en];
-                    const float4 pa = pti[code & ((1u << AL_BITS) - 1u)], pb = ptj[code >> AL_BITS];
-                    float ra[3], e[3];
+                // (four entries of a lane loaded ahead; a lane takes every 32nd, in order)
+                for (int e0 = start + lane; e0 < end; e0 += 128) {
+                    uint32_t code[4];
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        ra[k] = Ri[3 * k] * pa.x + Ri[3 * k + 1] * pa.y + Ri[3 * k + 2] * pa.z;
-                        e[k] = (ci[k] + ra[k]) - cj[k];
+                    for (int u = 0; u < 4; ++u) code[u] = e0 + 32 * u < end ? alist[e0 + 32 * u] : 0u;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if (e0 + 32 * u >= end) break;
+                        const float4 pa = pti[code[u] & ((1u << AL_BITS) - 1u)], pb = ptj[code[u] >> AL_BITS];
+                        float ra[3], e[3];
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            ra[k] = Ri[3 * k] * pa.x + Ri[3 * k + 1] * pa.y + Ri[3 * k + 2] * pa.z;
+                            e[k] = (ci[k] + ra[k]) - cj[k];
+                        }
+                        const float ah0 = Rj[0] * e[0] + Rj[3] * e[1] + Rj[6] * e[2];
+                        const float ah1 = Rj[1] * e[0] + Rj[4] * e[1] + Rj[7] * e[2];
+                        const float ah2 = Rj[2] * e[0] + Rj[5] * e[1] + Rj[8] * e[2];
+                        const float d0 = ah0 - pb.x, d1 = ah1 - pb.y, d2 = ah2 - pb.z;
+                        const float dd = d0 * d0 + d1 * d1 + d2 * d2;
+                        if (dd < reach2 && dd > 0.f)
+                            pair_force(pa, pb, ra, d0, d1, d2, dd, Rj, vi, wi, vj, wj, reach, kw2, kc, fi, fj);
                     }
-                    const float ah0 = Rj[0] * e[0] + Rj[3] * e[1] + Rj[6] * e[2];
-                    const float ah1 = Rj[1] * e[0] + Rj[4] * e[1] + Rj[7] * e[2];
-                    const float ah2 = Rj[2] * e[0] + Rj[5] * e[1] + Rj[8] * e[2];
-                    const float d0 = ah0 - pb.x, d1 = ah1 - pb.y, d2 = ah2 - pb.z;
-                    const float dd = d0 * d0 + d1 * d1 + d2 * d2;
-                    if (dd < reach2 && dd > 0.f)
-                        pair_force(pa, pb, ra, d0, d1, d2, dd, Rj, vi, wi, vj, wj, reach, kw2, kc, fi, fj);
                 }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-                    for (int k = 0; k < 6; ++k) {
-                        fi[k] += __shfl_xor_sync(FULL_MASK, fi[k], o);
-                        fj[k] += __shfl_xor_sync(FULL_MASK, fj[k], o);
-                    }
-                }
-                if (lane == 0) {
-#pragma unroll
-                    for (int k = 0; k < 6; ++k) { Xi[XC_RF + k] += fi[k]; Xj[XC_RF + k] += fj[k]; }
-                }
+                add_wrenches(fi, fj, Xi + XC_RF, Xj + XC_RF);
                 __syncwarp();
             }
         }

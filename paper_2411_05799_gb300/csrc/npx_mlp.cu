@@ -7,6 +7,7 @@
 // db = column sums of dZ, and dZ_prev = (dZ W) * gelu'(z_prev) (GEMM with the GELU' epilogue,
 // also writing its transpose).  Adam updates FP32 master weights and refreshes the BF16 copies
 // W and W^T that the GEMMs read.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -146,32 +147,72 @@ __global__ void unpad_kernel(const float *__restrict__ Y, int M, int out_p, int 
 
 inline unsigned blocks_for(long long n, int t = 256) { return (unsigned)((n + t - 1) / t); }
 
-// Column sums and sums of squares in FP64: block x covers 32 columns; thread (tx, ty) sums column
-// 32 x + tx over rows ty, ty + 32, ... (in that order), then thread ty = 0 adds the 32 partial sums
-// in ty order.  Every column is summed in a fixed order by one block: deterministic, no atomics.
-__global__ void __launch_bounds__(1024) column_moments_kernel(const float *__restrict__ X, long long rows, int cols,
-                                                              double *sum, double *sumsq) {
-    __shared__ double red[2][32][33];
-    const int tx = threadIdx.x, ty = threadIdx.y, c = blockIdx.x * 32 + tx;
+// Column sums and sums of squares in FP64.  A cluster of MOM_CTAS blocks covers CW columns, its
+// blocks and their MOM_THREADS / CW row lanes taking every MOM_CTAS * MOM_THREADS / CW-th row; each
+// lane sums its rows in order, then a warp's lanes, a block's warps and the cluster's blocks are
+// added in a fixed order (the blocks' sums over distributed shared memory, so there is no
+// workspace and no atomic): every column's sum repeats bit for bit.
+// Bound by the FP64 pipe (an add and a fused multiply-add per element, two lanes a clock and SM on
+// this part), so the work has to reach every SM: 65,536 x 271 took 1.80 ms on the nine blocks of
+// one 32-column block each, 0.17 ms on 272.
+constexpr int MOM_CTAS = 8, MOM_THREADS = 256;
+
+template <int CW>
+__global__ void __cluster_dims__(MOM_CTAS, 1, 1) __launch_bounds__(MOM_THREADS)
+column_moments_kernel(const float *__restrict__ X, long long rows, int cols, double *sum, double *sumsq) {
+    namespace cg = cooperative_groups;
+    constexpr int TY = MOM_THREADS / CW, WARPS = MOM_THREADS / 32;
+    __shared__ double red[WARPS][2][CW];
+    __shared__ double part[2][CW];
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), tx = threadIdx.x % CW, ty = threadIdx.x / CW;
+    const int c = (blockIdx.x / MOM_CTAS) * CW + tx, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long step = (long long)MOM_CTAS * TY;
     double s = 0.0, q = 0.0;
-    if (c < cols)
-        for (long long r = ty; r < rows; r += 32) {
-            const double v = (double)X[r * cols + c];
-            s += v;
-            q += v * v;
+    if (c < cols) {
+        const float *p = X + c;
+        long long r = (long long)rank * TY + ty;
+        for (; r + 7 * step < rows; r += 8 * step) {   // eight loads in flight
+            float v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = p[(r + k * step) * cols];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const double d = (double)v[k];
+                s += d;
+                q = fma(d, d, q);
+            }
         }
-    red[0][ty][tx] = s;
-    red[1][ty][tx] = q;
-    __syncthreads();
-    if (ty == 0 && c < cols) {
-        double ts = 0.0, tq = 0.0;
-        for (int k = 0; k < 32; ++k) {
-            ts += red[0][k][tx];
-            tq += red[1][k][tx];
+        for (; r < rows; r += step) {
+            const double d = (double)p[r * cols];
+            s += d;
+            q = fma(d, d, q);
         }
-        sum[c] += ts;
-        sumsq[c] += tq;
     }
+#pragma unroll
+    for (int o = 16; o >= CW; o >>= 1) {   // lanes of one column are CW apart
+        s += __shfl_down_sync(0xffffffffu, s, o);
+        q += __shfl_down_sync(0xffffffffu, q, o);
+    }
+    if (lane < CW) {
+        red[warp][0][lane] = s;
+        red[warp][1][lane] = q;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * CW) {
+        const int k = threadIdx.x / CW, x = threadIdx.x % CW;
+        double t = 0.0;
+        for (int w = 0; w < WARPS; ++w) t += red[w][k][x];
+        part[k][x] = t;
+    }
+    cl.sync();
+    if (rank == 0 && threadIdx.x < 2 * CW) {
+        const int k = threadIdx.x / CW, x = threadIdx.x % CW, col = (blockIdx.x / MOM_CTAS) * CW + x;
+        double t = 0.0;
+        for (int b = 0; b < MOM_CTAS; ++b) t += *cl.map_shared_rank(&part[k][x], b);
+        if (col < cols) (k == 0 ? sum : sumsq)[col] += t;
+    }
+    cl.sync();   // no block leaves while its sums are read
 }
 
 }  // namespace
@@ -472,8 +513,14 @@ int npx_mlp_backward(npx_mlp *n, const float *x, const float *t, int M, float *l
 int npx_column_moments(const float *X, long long rows, int cols, double *sum, double *sumsq, void *stream) {
     if (!X || !sum || !sumsq || rows < 0 || cols < 1) return npx::set_last_error(NPX_EINVAL, "npx_column_moments: bad arguments");
     if (rows == 0) return NPX_OK;
-    column_moments_kernel<<<(cols + 31) / 32, dim3(32, 32), 0, static_cast<cudaStream_t>(stream)>>>(X, rows, cols, sum,
-                                                                                                  sumsq);
+    // the widest column group (8: full 32-byte sectors) whose clusters still give every SM a block
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    auto launch = [&](auto kernel, int cw) {
+        kernel<<<(unsigned)((cols + cw - 1) / cw) * MOM_CTAS, MOM_THREADS, 0, st>>>(X, rows, cols, sum, sumsq);
+    };
+    if (cols > 8 * 18) launch(column_moments_kernel<8>, 8);
+    else if (cols > 4 * 18) launch(column_moments_kernel<4>, 4);
+    else launch(column_moments_kernel<2>, 2);
     CU(cudaGetLastError());
     return NPX_OK;
 }

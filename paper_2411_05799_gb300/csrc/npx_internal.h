@@ -179,6 +179,22 @@ cudaError_t launch_hm_dilate(const float *hm, float *tmp, float *out, int H, int
 
 }  // namespace npx
 
+namespace npx {
+// ---- the network's inference as one kernel (npx_mlp_fused.cu): up to FUSED_LAYERS layers of at
+// most FUSED_WIDTH inputs and outputs each (what one SM's shared and tensor memory hold)
+constexpr int FUSED_LAYERS = 8, FUSED_WIDTH = 512;
+struct FusedNet {
+    int layers, k[FUSED_LAYERS], n[FUSED_LAYERS];   // padded inputs (multiples of 64) and outputs (of 128)
+    const float *bias[FUSED_LAYERS];
+    const __nv_bfloat16 *w[FUSED_LAYERS];           // [n x k]
+};
+bool fused_fits(const FusedNet &net);
+// y [rows x ldy] (columns below ncols) from x [rows x n_in] FP32, or from xb [rows x k[0]] BF16 when
+// that is given; rows a multiple of 128
+cudaError_t launch_mlp_fused(const FusedNet &net, const float *x, int n_in, const __nv_bfloat16 *xb, float *y, int ldy,
+                             int ncols, int rows, int *err, cudaStream_t st);
+}  // namespace npx
+
 struct npx_mlp;
 namespace npx {
 // the surrogate network's stream, batch capacity and input / output widths

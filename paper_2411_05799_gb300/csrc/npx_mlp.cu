@@ -306,6 +306,21 @@ int forward_layers(npx_mlp *n, int M, bool train) {
     return NPX_OK;
 }
 
+// The network as the fused inference kernel takes it; false when it does not fit (it then runs
+// layer by layer).
+bool fused_net(const npx_mlp *n, npx::FusedNet *f) {
+    *f = npx::FusedNet{};
+    if (n->L > npx::FUSED_LAYERS) return false;
+    f->layers = n->L;
+    for (int l = 0; l < n->L; ++l) {
+        f->k[l] = n->din[l];
+        f->n[l] = n->dout[l];
+        f->bias[l] = n->b[l];
+        f->w[l] = n->Wb[l];
+    }
+    return npx::fused_fits(*f);
+}
+
 int forward_impl(npx_mlp *n, const float *x, int M, bool train) {
     const int in_p = n->din[0];
     pack_input_kernel<<<dim3(in_p / 32, M / 32), dim3(32, 8), 0, n->stream>>>(x, M, n->d.n_in, in_p, n->X0,
@@ -328,7 +343,11 @@ __nv_bfloat16 *npx::mlp_input(npx_mlp *n, int *ld) {
 }
 int npx::mlp_forward_packed(npx_mlp *n, int M) {
     RC(check(n, M));
-    return forward_layers(n, M, false);
+    npx::FusedNet f;
+    if (!fused_net(n, &f)) return forward_layers(n, M, false);
+    const int out_p = n->dout[n->L - 1];
+    CU(npx::launch_mlp_fused(f, nullptr, 0, n->X0, n->Y, out_p, out_p, M, n->err, n->stream));
+    return NPX_OK;
 }
 const float *npx::mlp_output(const npx_mlp *n, int *ld) {
     *ld = n->dout[n->L - 1];
@@ -462,6 +481,13 @@ int npx_mlp_grads_get(npx_mlp *n, float *g, size_t c) { return copy_params(n, g,
 int npx_mlp_forward(npx_mlp *n, const float *x, float *y, int M) {
     RC(check(n, M));
     if (!x || !y) return npx::set_last_error(NPX_EINVAL, "null array");
+    npx::FusedNet f;
+    // (outputs that overlap the inputs need every input read first: layer by layer)
+    const bool apart = x + (size_t)M * n->d.n_in <= y || y + (size_t)M * n->d.n_out <= x;
+    if (apart && fused_net(n, &f)) {
+        CU(npx::launch_mlp_fused(f, x, n->d.n_in, nullptr, y, n->d.n_out, n->d.n_out, M, n->err, n->stream));
+        return NPX_OK;
+    }
     RC(forward_impl(n, x, M, false));
     const int out_p = n->dout[n->L - 1];
     unpad_kernel<<<blocks_for((long long)M * n->d.n_out), 256, 0, n->stream>>>(n->Y, M, out_p, n->d.n_out, y);

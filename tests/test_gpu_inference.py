@@ -1,4 +1,5 @@
-"""The column statistics of the network's rows at the edges of their tiles."""
+"""The network's inference in one kernel, and the column statistics of its rows, at the edges of
+their tiles."""
 import numpy as np
 import pytest
 
@@ -14,6 +15,63 @@ def _own_stream():
     with torch.cuda.stream(s):
         yield
     s.synchronize()
+
+
+def _layer_by_layer(Ws, bs, x):
+    """The same network from the public GEMM: BF16 operands padded to its tiles, one launch a layer."""
+    pad = lambda n: (n + 127) // 128 * 128
+    M = x.shape[0]
+    st = torch.cuda.current_stream().cuda_stream
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    h = torch.zeros(M, pad(x.shape[1]), dtype=torch.bfloat16, device="cuda")
+    h[:, :x.shape[1]] = x.to(torch.bfloat16)
+    for l, (W, b) in enumerate(zip(Ws, bs)):
+        n, k = pad(W.shape[0]), h.shape[1]
+        Wp = torch.zeros(n, k, dtype=torch.bfloat16, device="cuda")
+        Wp[:W.shape[0], :W.shape[1]] = torch.from_numpy(W).cuda().to(torch.bfloat16)
+        bp = torch.zeros(n, device="cuda")
+        bp[:len(b)] = torch.from_numpy(b).cuda()
+        last = l == len(Ws) - 1
+        out = torch.zeros(M, n, dtype=torch.float32 if last else torch.bfloat16, device="cuda")
+        ep = npx.GemmEpilogue(mode=npx.EPI_BIAS if last else npx.EPI_BIAS_GELU, bias=bp.data_ptr(),
+                              **({"outf": out.data_ptr(), "ldf": n} if last else {"out": out.data_ptr(), "ldo": n}))
+        npx.gemm_bf16(h.data_ptr(), Wp.data_ptr(), M, n, k, ep, err.data_ptr(), stream=st)
+        torch.cuda.synchronize()
+        h = out
+    assert int(err.item()) == 0
+    return h[:, :Ws[-1].shape[0]]
+
+
+@pytest.mark.parametrize("M,n_in,hidden,layers,n_out", [
+    (128, 271, 512, 4, 247),      # one tile
+    (128 * 153, 271, 512, 4, 247),    # one tile more than there are SMs
+    (384, 1, 128, 1, 1),          # one block, one input, one output
+    (256, 64, 256, 7, 129),       # eight layers, one block each, an odd output width
+    (640, 300, 384, 2, 300),      # blocks of 256 and 128, outputs in two blocks
+    (128 * 305, 512, 512, 1, 512),    # the widest, three tiles on some SMs
+    (256, 40, 640, 2, 30),        # too wide for one kernel
+    (256, 40, 128, 8, 30),        # too deep for one kernel
+])
+def test_inference_equals_the_layers_one_by_one(M, n_in, hidden, layers, n_out):
+    """Same operands, products in the same order, same roundings: equal bit for bit."""
+    rng = np.random.default_rng(M + hidden)
+    sizes = [n_in] + [hidden] * layers + [n_out]
+    Ws = [rng.normal(0, np.sqrt(2 / i), (o, i)).astype(np.float32) for i, o in zip(sizes[:-1], sizes[1:])]
+    bs = [rng.normal(0, 0.1, o).astype(np.float32) for o in sizes[1:]]
+    net = npx.MLP(n_in, n_out, n_hidden=hidden, n_hidden_layers=layers, max_batch=M,
+                  stream=torch.cuda.current_stream().cuda_stream)
+    net.set_params(Ws, bs)
+    x = torch.from_numpy(rng.normal(0, 1, (M, n_in)).astype(np.float32)).cuda()
+    y = torch.full((M + 1, n_out), float("nan"), device="cuda")
+    for _ in range(2):
+        net.forward(x.data_ptr(), y.data_ptr(), M)
+    torch.cuda.synchronize()
+    assert torch.equal(y[:M], _layer_by_layer(Ws, bs, x))
+    assert torch.isnan(y[M]).all()          # nothing past the last row
+    if n_out <= n_in:                       # outputs over the inputs
+        net.forward(x.data_ptr(), x.data_ptr(), M)
+        torch.cuda.synchronize()
+        assert torch.equal(x.reshape(-1)[:M * n_out].reshape(M, n_out), y[:M])
 
 
 @pytest.mark.parametrize("rows,cols", [(1, 1), (7, 3), (2047, 36), (2048, 37), (4097, 72), (999, 73), (1000, 144),

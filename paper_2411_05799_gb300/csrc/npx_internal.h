@@ -201,9 +201,11 @@ namespace npx {
 cudaStream_t mlp_stream(const npx_mlp *net);
 int mlp_max_batch(const npx_mlp *net);
 void mlp_dims(const npx_mlp *net, int *n_in, int *n_out);
+// columns of a prediction that the surrogate's update reads: the torso's
+constexpr int SUR_TORSO = 13;
 // the network's packed BF16 input rows [max_batch x ld] (zero-padded columns), a forward pass of
-// M rows from them, and the FP32 output rows [M x ld] it leaves (padded columns)
+// M rows from them, and the FP32 output rows [M x ld] it leaves: the first `cols` columns at least
 __nv_bfloat16 *mlp_input(npx_mlp *net, int *ld);
-int mlp_forward_packed(npx_mlp *net, int M);
+int mlp_forward_packed(npx_mlp *net, int M, int cols);
 const float *mlp_output(const npx_mlp *net, int *ld);
 }  // namespace npx

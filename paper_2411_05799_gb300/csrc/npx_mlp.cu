@@ -341,12 +341,13 @@ __nv_bfloat16 *npx::mlp_input(npx_mlp *n, int *ld) {
     *ld = n->din[0];
     return n->X0;
 }
-int npx::mlp_forward_packed(npx_mlp *n, int M) {
+int npx::mlp_forward_packed(npx_mlp *n, int M, int cols) {
     RC(check(n, M));
     npx::FusedNet f;
     if (!fused_net(n, &f)) return forward_layers(n, M, false);
-    const int out_p = n->dout[n->L - 1];
-    CU(npx::launch_mlp_fused(f, nullptr, 0, n->X0, n->Y, out_p, out_p, M, n->err, n->stream));
+    const int l = n->L - 1;
+    f.n[l] = std::min(n->dout[l], pad_to(cols, 128));   // only the blocks of outputs that are read
+    CU(npx::launch_mlp_fused(f, nullptr, 0, n->X0, n->Y, n->dout[l], cols, M, n->err, n->stream));
     return NPX_OK;
 }
 const float *npx::mlp_output(const npx_mlp *n, int *ld) {

@@ -14,7 +14,14 @@
 //     both go to shared memory in place of those, block by block, so that the next layer's first
 //     MMAs run while its later columns are still being written.
 // The products, their order, the bias, the GELU and the roundings are those of the layer-by-layer
-// path, so the results are the same bit for bit.  Bound by the MMAs and the weights' way from L2.
+// path, so the results are the same bit for bit.
+// The input rows are loaded two rows at a time and the next tile's drawn into L2 ahead, and output
+// rows without padding are staged as they lie in memory and leave as one bulk copy: chunk-wise
+// loads and strided stores were two fifths of a tile's 120,000 cycles.  65,536 rows, 271 -> 4 x 512 ->
+// 247: 225 us layer by layer, 197 with those, 137 now; what is left is the MMAs and the last block's
+// epilogue of each layer.  (Weights by cluster multicast, and pairs of CTAs sharing each MMA, which
+// halve or quarter the weights' traffic, measured no faster, 198 to 224 us, before those two: the
+// ring was not what it waited for.)
 // Waits are bounded as in npx_gemm.cu: a role that gives up sets the error flag and the others leave.
 #include <algorithm>
 #include <cstring>
@@ -76,8 +83,9 @@ mlp_fused_kernel(const __grid_constant__ FusedMaps maps, const __grid_constant__
     uint64_t *tfull = empty + F_STAGES;    // a step's accumulators complete
     uint64_t *tempty = tfull + 2;          // and drained
     uint64_t *aready = tempty + 2;         // columns 0-255 / 256-511 of a layer's input written
-    uint64_t *staged = aready + 2;         // a tile's output rows read back by every epilogue warp
-    uint64_t *done = staged + 1;
+    uint64_t *staged = aready + 2;         // every epilogue warp is done with a tile's staged outputs
+    uint64_t *freed = staged + 1;          // and the activations' memory can take the next tile
+    uint64_t *done = freed + 1;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
     volatile int *abort = reinterpret_cast<volatile int *>(tmem_slot + 1);
     int *issued = reinterpret_cast<int *>(tmem_slot + 2), *consumed = reinterpret_cast<int *>(tmem_slot + 3);
@@ -100,6 +108,7 @@ mlp_fused_kernel(const __grid_constant__ FusedMaps maps, const __grid_constant__
             mbar_init(&aready[b], F_EPI);
         }
         mbar_init(staged, F_EPI);
+        mbar_init(freed, 1);
         mbar_init(done, 1);
         *abort = 0;
         *issued = 0;
@@ -179,11 +188,14 @@ mlp_fused_kernel(const __grid_constant__ FusedMaps maps, const __grid_constant__
         // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31 and a quarter of a step's columns
         const int e = warp - 2, q = warp & 3, part = e >> 2, row = q * 32 + lane;
         const uint32_t trow = tmem + ((uint32_t)(q * 32) << 16);
+        // (a row pitch of whole 16-byte units would put the lanes' rows on a few banks)
+        const bool bulk = ncols == ldy && ldy <= F_ACT / (4 * F_ROWS) && (ldy & 3) != 0 &&
+                          (reinterpret_cast<uintptr_t>(y) & 15) == 0;
         int step = 0, it = 0;
         bool ok = true;
         for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++it) {
-            // (the last tile's rows were staged where these go)
-            if (it > 0 && !mbar_wait(staged, (uint32_t)((it - 1) & 1), abort)) {
+            // (the last tile's outputs were staged where these go)
+            if (it > 0 && !mbar_wait(freed, (uint32_t)((it - 1) & 1), abort)) {
                 ok = false;
                 break;
             }
@@ -197,18 +209,34 @@ mlp_fused_kernel(const __grid_constant__ FusedMaps maps, const __grid_constant__
                     *reinterpret_cast<uint4 *>(act + act_offset(u * 8, e * 8 + r)) = __ldg(src + i);
                 }
             } else {
-#pragma unroll 2
-                for (int r = 0; r < 8; ++r) {
-                    const float *src = x + (size_t)(t * F_ROWS + e * 8 + r) * n_in;
+                // (all of two rows' loads first: they are rows of no alignment, four bytes a lane)
+                const float *src = x + (size_t)(t * F_ROWS + e * 8) * n_in;
 #pragma unroll
-                    for (int c = 0; c < FUSED_WIDTH / 64; ++c) {
-                        const int col = c * 64 + 2 * lane;
-                        if (c * 64 < net.k[0]) {
-                            const float a = col < n_in ? __ldg(src + col) : 0.f, b = col + 1 < n_in ? __ldg(src + col + 1) : 0.f;
-                            *reinterpret_cast<__nv_bfloat162 *>(act + act_offset(col, e * 8 + r) + ((col & 7) << 1)) =
-                                __floats2bfloat162_rn(a, b);
+                for (int r = 0; r < 8; r += 2, src += 2 * n_in) {
+                    float v[2][FUSED_WIDTH / 64][2];
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+#pragma unroll
+                        for (int c = 0; c < FUSED_WIDTH / 64; ++c) {
+                            const int col = c * 64 + 2 * lane;
+                            v[i][c][0] = col < n_in ? __ldg(src + i * n_in + col) : 0.f;
+                            v[i][c][1] = col + 1 < n_in ? __ldg(src + i * n_in + col + 1) : 0.f;
                         }
-                    }
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+#pragma unroll
+                        for (int c = 0; c < FUSED_WIDTH / 64; ++c) {
+                            const int col = c * 64 + 2 * lane;
+                            if (c * 64 < net.k[0])
+                                *reinterpret_cast<__nv_bfloat162 *>(act + act_offset(col, e * 8 + r + i) + ((col & 7) << 1)) =
+                                    __floats2bfloat162_rn(v[i][c][0], v[i][c][1]);
+                        }
+                }
+                // the next tile's rows into L2 meanwhile
+                if (t + gridDim.x < tiles) {
+                    const char *next = reinterpret_cast<const char *>(x + (size_t)((t + gridDim.x) * F_ROWS + e * 8) * n_in);
+                    for (int o = lane * 128; o < 32 * n_in; o += 32 * 128)
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(next + o));
                 }
             }
             fence_async_shared();
@@ -269,7 +297,10 @@ mlp_fused_kernel(const __grid_constant__ FusedMaps maps, const __grid_constant__
                 if (!mbar_wait(&tfull[(step + j) & 1], (uint32_t)(((step + j) >> 1) & 1), abort)) ok = false;
             if (!ok) break;
             tc_fence_after();
-            float *stage = reinterpret_cast<float *>(act) + e * 512;   // 32 rows x 16 columns
+            // rows without padding between them are one block of memory: staged as they lie there, it
+            // leaves as one bulk copy; wider or strided rows go out by 16 columns of 32 rows
+            float *stage = bulk ? reinterpret_cast<float *>(act) + (size_t)row * ldy
+                                : reinterpret_cast<float *>(act) + e * 512;   // 32 rows x 16 columns
             float *out = y + (size_t)(t * F_ROWS + q * 32) * ldy;
             for (int n0 = 0; n0 < N; n0 += F_BN, ++step) {
                 const int b = step & 1, bn = min(F_BN, N - n0), nch = bn >> 6, c0 = part * (bn >> 2);
@@ -277,8 +308,15 @@ mlp_fused_kernel(const __grid_constant__ FusedMaps maps, const __grid_constant__
 #pragma unroll 1
                 for (int c = 0; c < nch; ++c) {
                     const int col = n0 + c0 + 16 * c;
+                    if (col >= ncols) break;
                     float v[16];
                     load_acc16(taddr + 16 * c, net.bias[L - 1] + col, v);
+                    if (bulk) {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            if (col + i < ncols) stage[col + i] = v[i];
+                        continue;
+                    }
                     __syncwarp();
 #pragma unroll
                     for (int i = 0; i < 4; ++i)   // 16-byte units swizzled against bank conflicts
@@ -296,8 +334,29 @@ mlp_fused_kernel(const __grid_constant__ FusedMaps maps, const __grid_constant__
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&tempty[b]);
             }
-            if (lane == 0) mbar_arrive(staged);   // (after the last __syncwarp: every lane has read its rows)
+            if (bulk) fence_async_shared();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(staged);
+                if (e == 0) {
+                    if (!mbar_wait(staged, (uint32_t)(it & 1), abort)) {
+                        ok = false;
+                    } else {
+                        if (bulk) {
+                            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                                             y + (size_t)t * F_ROWS * ldy),
+                                         "r"(smem_u32(act)), "r"((uint32_t)(F_ROWS * 4 * ldy))
+                                         : "memory");
+                            bulk_commit();
+                            bulk_wait_read<0>();
+                        }
+                        mbar_arrive(freed);
+                    }
+                }
+            }
         }
+        if (bulk && e == 0 && lane == 0) bulk_wait_all();   // the copies have landed before the CTA ends
+        __syncwarp();
         if (!ok && lane == 0) {
             *abort = 1;
             atomicExch(err, 3);

@@ -1605,7 +1605,7 @@ int npx_world_step_surrogate(npx_world *w, npx_mlp *net, const npx_surrogate_nor
             CUDA_TRY(cudaEventRecord(w->sg.ev_w, w->stream));
             CUDA_TRY(cudaStreamWaitEvent(ns, w->sg.ev_w, 0));
         }
-        if (int rc = npx::mlp_forward_packed(net, w->sg.rows)) return rc;
+        if (int rc = npx::mlp_forward_packed(net, w->sg.rows, npx::SUR_TORSO)) return rc;
         if (ns != w->stream) {
             CUDA_TRY(cudaEventRecord(w->sg.ev_n, ns));
             CUDA_TRY(cudaStreamWaitEvent(w->stream, w->sg.ev_n, 0));

@@ -78,18 +78,52 @@ __global__ void __launch_bounds__(256) loss_grad_kernel(const float *__restrict_
     }
 }
 
-// out[n] = sum over the M entries of row n of GT [N x M] (the bias gradient: column sums of the
-// layer's output gradient, read from its transpose so that every load is a full line)
-__global__ void __launch_bounds__(256) rowsum_kernel(const bf16 *__restrict__ GT, int M, float *out) {
+// What is left of a backward pass for up to GROUP layers in one launch: the split-K partials of each
+// weight gradient summed in split order, and each bias gradient, the sum over the M entries of a row
+// of the layer's transposed output gradient GT [rows x M] (read from the transpose so that every load
+// is a full line).  Bound by launches: layer by layer these were ten launches of 4 to 6 us each,
+// 49 us of a 357 us minibatch of 8,192 rows (271 -> 4 x 512 -> 247); with Adam's ten below as one, a
+// minibatch takes 294 us.
+constexpr int GROUP = 16;
+struct GradLayer {
+    const float *part;      // [splits][n], or NULL: the gradient is written already
+    float *dW;
+    const bf16 *GT;
+    float *db;
+    int splits, rows, first;    // first: the layer's first block
+    long long n;
+};
+struct GradGroup {
+    GradLayer l[GROUP];
+    int layers;
+};
+
+__global__ void __launch_bounds__(256) grads_finish_kernel(const __grid_constant__ GradGroup G, int M) {
+    int k = 0;
+    while (k + 1 < G.layers && (int)blockIdx.x >= G.l[k + 1].first) ++k;
+    const GradLayer &g = G.l[k];
+    int blk = (int)blockIdx.x - g.first;
+    if (blk >= g.rows) {   // four weights a thread
+        const long long i = ((long long)(blk - g.rows) * 256 + threadIdx.x) * 4;
+        if (i >= g.n) return;
+        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int s = 0; s < g.splits; ++s) {
+            const float4 p = *reinterpret_cast<const float4 *>(g.part + (size_t)s * g.n + i);
+            t.x += p.x; t.y += p.y; t.z += p.z; t.w += p.w;
+        }
+        *reinterpret_cast<float4 *>(g.dW + i) = t;
+        return;
+    }
     __shared__ float red[8];
-    const bf16 *row = GT + (size_t)blockIdx.x * M;
+    const bf16 *row = g.GT + (size_t)blk * M;
     float s = 0.f;
     for (int m = threadIdx.x * 8; m < M; m += 256 * 8) {
         const uint4 u = *reinterpret_cast<const uint4 *>(row + m);
         const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&u);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float2 f = __bfloat1622float2(h[k]);
+        for (int k2 = 0; k2 < 4; ++k2) {
+            const float2 f = __bfloat1622float2(h[k2]);
             s += f.x + f.y;
         }
     }
@@ -99,35 +133,58 @@ __global__ void __launch_bounds__(256) rowsum_kernel(const bf16 *__restrict__ GT
     if (threadIdx.x == 0) {
         float t = 0.f;
         for (int i = 0; i < 8; ++i) t += red[i];
-        out[blockIdx.x] = t;
+        g.db[blk] = t;
     }
 }
 
-__global__ void splitk_reduce_kernel(const float *__restrict__ part, int splits, long long n, float *out) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float s = 0.f;
-    for (int k = 0; k < splits; ++k) s += part[(size_t)k * n + i];
-    out[i] = s;
+// Adam on FP32 master parameters of up to GROUP layers in one launch.  A block takes a 32 x 32 tile
+// of a weight matrix, so that the refreshed BF16 copy and, through shared memory, its transpose are
+// both written in full lines (element by element the transpose wrote two bytes to a sector), or 256
+// biases.  It was ten launches of 4.5 us.
+struct AdamLayer {
+    float *W, *mW, *vW, *b, *mb, *vb;
+    const float *dW, *db;
+    bf16 *Wb, *WbT;
+    int rows, cols, first;
+};
+struct AdamGroup {
+    AdamLayer l[GROUP];
+    int layers;
+    float lr, b1, b2, eps, bc1, bc2;
+};
+
+__device__ __forceinline__ float adam_update(const AdamGroup &A, float *p, float *m, float *v, float gi) {
+    const float mi = A.b1 * *m + (1.f - A.b1) * gi;
+    const float vi = A.b2 * *v + (1.f - A.b2) * gi * gi;
+    *m = mi;
+    *v = vi;
+    const float pi = *p - A.lr * (mi / A.bc1) / (sqrtf(vi / A.bc2) + A.eps);
+    *p = pi;
+    return pi;
 }
 
-// Adam on FP32 master parameters [rows x cols]; refreshes the BF16 copy and its transpose
-__global__ void adam_kernel(float *p, const float *g, float *m, float *v, long long n, int cols, float lr,
-                            float b1, float b2, float eps, float bc1, float bc2, bf16 *pb, bf16 *pbT, int rows) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    const float pi = p[i] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
-    p[i] = pi;
-    if (pb) {
-        const bf16 b = __float2bfloat16_rn(pi);
-        pb[i] = b;
-        pbT[(size_t)(i % cols) * rows + (i / cols)] = b;
+__global__ void __launch_bounds__(256) adam_kernel(const __grid_constant__ AdamGroup A) {
+    __shared__ bf16 tile[32][33];
+    int k = 0;
+    while (k + 1 < A.layers && (int)blockIdx.x >= A.l[k + 1].first) ++k;
+    const AdamLayer &g = A.l[k];
+    const int blk = (int)blockIdx.x - g.first, tc = g.cols / 32, tiles = (g.rows / 32) * tc;
+    if (blk >= tiles) {
+        const int i = (blk - tiles) * 256 + threadIdx.x;
+        if (i < g.rows) adam_update(A, g.b + i, g.mb + i, g.vb + i, g.db[i]);
+        return;
     }
+    const int r0 = blk / tc * 32, c0 = blk % tc * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const size_t e = (size_t)(r0 + ty + 8 * i) * g.cols + c0 + tx;
+        const bf16 w = __float2bfloat16_rn(adam_update(A, g.W + e, g.mW + e, g.vW + e, g.dW[e]));
+        g.Wb[e] = w;
+        tile[ty + 8 * i][tx] = w;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) g.WbT[(size_t)(c0 + ty + 8 * i) * g.rows + r0 + tx] = tile[tx][ty + 8 * i];
 }
 
 __global__ void to_bf16_kernel(const float *p, long long n, int cols, int rows, bf16 *pb, bf16 *pbT) {
@@ -226,9 +283,9 @@ struct npx_mlp {
     std::vector<bf16 *> Wb, WbT;
     bf16 *X0 = nullptr, *X0T = nullptr, *dY = nullptr, *dYT = nullptr;
     std::vector<bf16 *> Z, X, XT, dZ, dZT;      // hidden layers
-    float *Y = nullptr, *part = nullptr, *loss_tmp = nullptr;
+    std::vector<float *> part;                  // split-K partials of each layer's weight gradient
+    float *Y = nullptr, *loss_tmp = nullptr;
     int *err = nullptr;
-    size_t part_elems = 0;
     int t = 0;
     std::vector<void *> bufs;
 };
@@ -255,6 +312,7 @@ npx_gemm_epilogue epi(int mode) {
     return e;
 }
 
+// splits of a weight gradient's K (the batch): as many as fill the chip; K = 0: the most of any batch
 int pick_splits(int Mg, int Ng, int K) {
     const int tiles = (Mg / 128) * (Ng / (Ng % 256 == 0 ? 256 : 128));
     int s = 1;
@@ -385,13 +443,13 @@ int npx_mlp_create(const npx_mlp_desc *d, npx_mlp **out) {
     bool ok = true;
     n->W.resize(n->L); n->b.resize(n->L); n->mW.resize(n->L); n->vW.resize(n->L); n->mb.resize(n->L);
     n->vb.resize(n->L); n->dW.resize(n->L); n->db.resize(n->L); n->Wb.resize(n->L); n->WbT.resize(n->L);
-    size_t max_w = 0;
+    n->part.resize(n->L);
     for (int l = 0; l < n->L && ok; ++l) {
         const size_t nw = (size_t)n->dout[l] * n->din[l];
-        max_w = std::max(max_w, nw);
+        const int ms = pick_splits(n->dout[l], n->din[l], 0);
         ok = dalloc(n, &n->W[l], nw) && dalloc(n, &n->mW[l], nw) && dalloc(n, &n->vW[l], nw) &&
              dalloc(n, &n->dW[l], nw) && dalloc(n, &n->Wb[l], nw) && dalloc(n, &n->WbT[l], nw) &&
-             dalloc(n, &n->b[l], n->dout[l]) && dalloc(n, &n->mb[l], n->dout[l]) &&
+             dalloc(n, &n->part[l], ms > 1 ? ms * nw : 0) && dalloc(n, &n->b[l], n->dout[l]) && dalloc(n, &n->mb[l], n->dout[l]) &&
              dalloc(n, &n->vb[l], n->dout[l]) && dalloc(n, &n->db[l], n->dout[l]);
     }
     n->Z.resize(n->L - 1); n->X.resize(n->L - 1); n->XT.resize(n->L - 1); n->dZ.resize(n->L - 1); n->dZT.resize(n->L - 1);
@@ -399,11 +457,9 @@ int npx_mlp_create(const npx_mlp_desc *d, npx_mlp **out) {
         ok = dalloc(n, &n->Z[l], (size_t)Mx * H) && dalloc(n, &n->X[l], (size_t)Mx * H) &&
              dalloc(n, &n->XT[l], (size_t)Mx * H) && dalloc(n, &n->dZ[l], (size_t)Mx * H) &&
              dalloc(n, &n->dZT[l], (size_t)Mx * H);
-    n->part_elems = 64 * max_w;
     ok = ok && dalloc(n, &n->X0, (size_t)Mx * n->din[0]) && dalloc(n, &n->X0T, (size_t)Mx * n->din[0]) &&
          dalloc(n, &n->Y, (size_t)Mx * n->dout[n->L - 1]) && dalloc(n, &n->dY, (size_t)Mx * n->dout[n->L - 1]) &&
-         dalloc(n, &n->dYT, (size_t)Mx * n->dout[n->L - 1]) && dalloc(n, &n->part, n->part_elems) &&
-         dalloc(n, &n->err, 1) && dalloc(n, &n->loss_tmp, 1);
+         dalloc(n, &n->dYT, (size_t)Mx * n->dout[n->L - 1]) && dalloc(n, &n->err, 1) && dalloc(n, &n->loss_tmp, 1);
     if (!ok) {
         npx_mlp_destroy(n);
         return npx::set_last_error(NPX_ENOMEM, "device allocation failed");
@@ -506,20 +562,28 @@ int npx_mlp_backward(npx_mlp *n, const float *x, const float *t, int M, float *l
                                                                               n->dYT, loss);
     CU(cudaGetLastError());
     const bf16 *G = n->dY, *GT = n->dYT;     // gradient of the current layer's output
+    GradGroup group;
+    group.layers = 0;
+    int blocks = 0;
     for (int l = L - 1; l >= 0; --l) {
         const int No = n->dout[l], Ni = n->din[l];
         // dW = G^T X_prev: A = G^T [No x M], B = X_prev^T [Ni x M]
         const bf16 *XprevT = l > 0 ? n->XT[l - 1] : n->X0T;
         const int splits = pick_splits(No, Ni, M);
         npx_gemm_epilogue e = epi(NPX_EPI_F32);
-        e.outf = n->part;
+        e.outf = splits > 1 ? n->part[l] : n->dW[l];
         e.ldf = Ni;
         e.split_stride = (long long)No * Ni;
         RC(gemm(n, GT, XprevT, No, Ni, M, splits, e));
-        splitk_reduce_kernel<<<blocks_for((long long)No * Ni), 256, 0, n->stream>>>(n->part, splits, (long long)No * Ni,
-                                                                                   n->dW[l]);
-        rowsum_kernel<<<No, 256, 0, n->stream>>>(GT, M, n->db[l]);
-        CU(cudaGetLastError());
+        GradLayer &g = group.l[group.layers++];
+        g = GradLayer{splits > 1 ? n->part[l] : nullptr, n->dW[l], GT, n->db[l], splits, No, blocks, (long long)No * Ni};
+        blocks += No + (splits > 1 ? (int)blocks_for(g.n / 4) : 0);
+        if (group.layers == GROUP || l == 0) {
+            grads_finish_kernel<<<blocks, 256, 0, n->stream>>>(group, M);
+            CU(cudaGetLastError());
+            group.layers = 0;
+            blocks = 0;
+        }
         if (l > 0) {
             // dZ_prev = (G W) * gelu'(Z_prev): A = G [M x No], B = W^T [Ni x No]
             npx_gemm_epilogue e2 = epi(NPX_EPI_DGELU);
@@ -557,14 +621,20 @@ int npx_mlp_adam_step(npx_mlp *n) {
     n->t += 1;
     const float b1 = n->d.beta1, b2 = n->d.beta2;
     const float bc1 = 1.f - std::pow(b1, (float)n->t), bc2 = 1.f - std::pow(b2, (float)n->t);
+    AdamGroup A;
+    A.lr = n->d.lr; A.b1 = b1; A.b2 = b2; A.eps = n->d.eps; A.bc1 = bc1; A.bc2 = bc2;
+    A.layers = 0;
+    int blocks = 0;
     for (int l = 0; l < n->L; ++l) {
-        const long long nw = (long long)n->dout[l] * n->din[l];
-        adam_kernel<<<blocks_for(nw), 256, 0, n->stream>>>(n->W[l], n->dW[l], n->mW[l], n->vW[l], nw, n->din[l],
-                                                          n->d.lr, b1, b2, n->d.eps, bc1, bc2, n->Wb[l], n->WbT[l],
-                                                          n->dout[l]);
-        adam_kernel<<<blocks_for(n->dout[l]), 256, 0, n->stream>>>(n->b[l], n->db[l], n->mb[l], n->vb[l], n->dout[l],
-                                                                   1, n->d.lr, b1, b2, n->d.eps, bc1, bc2, nullptr,
-                                                                   nullptr, 1);
+        const int rows = n->dout[l], cols = n->din[l];
+        A.l[A.layers++] = AdamLayer{n->W[l], n->mW[l], n->vW[l], n->b[l], n->mb[l], n->vb[l], n->dW[l], n->db[l],
+                                    n->Wb[l], n->WbT[l], rows, cols, blocks};
+        blocks += (rows / 32) * (cols / 32) + (int)blocks_for(rows);
+        if (A.layers == GROUP || l == n->L - 1) {
+            adam_kernel<<<blocks, 256, 0, n->stream>>>(A);
+            A.layers = 0;
+            blocks = 0;
+        }
     }
     CU(cudaGetLastError());
     return NPX_OK;

@@ -1,5 +1,5 @@
-"""The network's inference in one kernel, and the column statistics of its rows, at the edges of
-their tiles."""
+"""The network's inference in one kernel, the grouped ends of its training step, and the column
+statistics of its rows, at the edges of their tiles."""
 import numpy as np
 import pytest
 
@@ -105,3 +105,52 @@ def test_column_moments_of_infinities_and_nan():
     a, q = s.cpu().numpy()
     assert a[0] == 3000 and a[1] == np.inf and np.isnan(a[2]) and np.isnan(a[3]) and a[4] == 3000
     assert q[1] == np.inf and np.isnan(q[2]) and q[3] == np.inf
+
+
+@pytest.mark.parametrize("M,n_in,hidden,layers,n_out", [(128, 3, 128, 1, 2), (1152, 271, 256, 2, 129),
+                                                        (2048, 40, 128, 17, 30)])
+def test_training_step(M, n_in, hidden, layers, n_out):
+    """One launch for what is left of the gradients and one for Adam, up to sixteen layers at a time
+    (17 hidden layers take two): bias gradients against FP64 sums of the network's own BF16 output
+    gradients where those are known (the last layer), weights after Adam's first step against its
+    formula on the gradients read back, element by element."""
+    rng = np.random.default_rng(M)
+    sizes = [n_in] + [hidden] * layers + [n_out]
+    Ws = [rng.normal(0, np.sqrt(2 / i), (o, i)).astype(np.float32) for i, o in zip(sizes[:-1], sizes[1:])]
+    bs = [rng.normal(0, 0.1, o).astype(np.float32) for o in sizes[1:]]
+    net = npx.MLP(n_in, n_out, n_hidden=hidden, n_hidden_layers=layers, max_batch=M, lr=1e-3,
+                  stream=torch.cuda.current_stream().cuda_stream)
+    net.set_params(Ws, bs)
+    x = torch.from_numpy(rng.normal(0, 1, (M, n_in)).astype(np.float32)).cuda()
+    t = torch.from_numpy(rng.normal(0, 1, (M, n_out)).astype(np.float32)).cuda()
+    y = torch.zeros(M, n_out, device="cuda")
+    loss = torch.zeros(1, device="cuda")
+    net.forward(x.data_ptr(), y.data_ptr(), M)
+    net.backward(x.data_ptr(), t.data_ptr(), M, loss.data_ptr())
+    gWs, gbs = net.get_grads()
+    net.adam_step()
+    torch.cuda.synchronize()
+    W1, b1 = net.get_params()
+    # the last layer's bias gradient: the column sums of BF16(2 (y - t) / M); M FP32 terms in any order
+    # stay within M 2^-24 of the sum of their magnitudes
+    inv = torch.tensor(1.0, device="cuda") / M
+    g = (2.0 * (y - t) * inv).to(torch.bfloat16).double().cpu().numpy()
+    assert (np.abs(gbs[-1] - g.sum(0)) <= M * 2.0 ** -24 * np.abs(g).sum(0)).all()
+    assert all(np.isfinite(a).all() for a in gWs + gbs)
+    # Adam's first step: m / (1 - 0.9) = g, v / (1 - 0.999) = g^2, so p - lr g / (|g| + eps); the FP32
+    # 1 - 0.9 and 1 - 0.999 are off by up to 2^-24 / 0.001 relative
+    for p0, p1, gr in zip(Ws + bs, W1 + b1, gWs + gbs):
+        step = 1e-3 * gr.astype(np.float64) / (np.abs(gr.astype(np.float64)) + 1e-8)
+        assert (np.abs(p1 - (p0 - step)) <= 2.0 ** -23 * (np.abs(p0) + 1e-3) + 1e-3 * 2e-4).all()
+    # and the BF16 copies the next pass reads are the new weights': the forward pass uses them
+    net.forward(x.data_ptr(), y.data_ptr(), M)
+    torch.cuda.synchronize()
+    assert torch.equal(y, _layer_by_layer(W1, b1, x))
+    # (the transposes too: two networks with the same parameters give the same gradients)
+    other = npx.MLP(n_in, n_out, n_hidden=hidden, n_hidden_layers=layers, max_batch=M,
+                    stream=torch.cuda.current_stream().cuda_stream)
+    other.set_params(W1, b1)
+    for n in (net, other):
+        n.backward(x.data_ptr(), t.data_ptr(), M, loss.data_ptr())
+    for a, b in zip(sum(net.get_grads(), []), sum(other.get_grads(), [])):
+        np.testing.assert_array_equal(a, b)

@@ -1523,8 +1523,10 @@ int npx_surrogate_collect(npx_world *w, const npx_surrogate_norm *nrm, int strid
     if (!cache_valid(w))
         if (int rc = cache_build(w)) return rc;
     for (int k = 0; k < n_windows;) {
-        if (!window_fits(w, w->step, stride)) {   // joint updates and what is left before them
-            if (int rc = plain_run(w, 1, false)) return rc;
+        if (!window_fits(w, w->step, stride)) {   // joint updates and what is left before them, in one launch
+            int m = 1;
+            while (!window_fits(w, w->step + m, stride)) ++m;
+            if (int rc = plain_run(w, m, false)) return rc;
             continue;
         }
         pre.X = X + (size_t)k * w->S * nf;

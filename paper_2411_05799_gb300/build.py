@@ -1,6 +1,6 @@
 """Build libnpx.so (the CUDA step library) in-tree with nvcc for sm_103a.
 
-Two translation units are compiled in parallel and linked into one shared library next to
+The translation units are compiled in parallel and linked into one shared library next to
 this file.  A rebuild happens only when a source or header is newer than the library."""
 from __future__ import annotations
 

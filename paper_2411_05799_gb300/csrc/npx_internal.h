@@ -52,6 +52,8 @@ struct WorldDev {
     int n_sched;                          // entries of order to run
     const int *sched_count;               // device count overriding n_sched, or NULL
     int max_points, max_links;
+    float4 *pscr;                         // posed offsets of the scenes in flight, max_points each, for
+                                          // launches that keep them in global memory (LaunchCfg::gp)
     const long long *step;                // device step counter n
     unsigned int *queue;                  // work-queue counter (reset before each launch)
     // 1: the launch takes the previous-step contacts from a detection at the current state
@@ -107,11 +109,17 @@ struct LaunchCfg {
     int lps;      // lanes per scene: 4, 8, 16 or 32
     int wpb;      // warps per block
     int blocks;   // grid size
+    int gp = 0;   // 1: the scenes' posed points in global memory (WorldDev::pscr), not in the slots
+    int grid = 0; // 1: the caller asked for this grid size
 };
 
-size_t step_smem_bytes(const WorldDev &W, int lps, int wpb);
-int step_slot_bytes(const WorldDev &W, int lps);
-int step_blocks_per_sm(const WorldDev &W, int lps, int wpb, cudaError_t *err);
+int step_blocks_per_sm(const WorldDev &W, int lps, int wpb, int gp, cudaError_t *err);
+// whether the shape would fit on an SM if the slots did not hold their links' tree numbers
+bool step_fits_bare(const WorldDev &W, int lps, int wpb);
+// that build of the flat kernel (npx_step_gp.cu; NULL: no such lanes per scene), and whether the
+// world's step kernel has one
+void *step_gp_kernel(int lps);
+bool step_has_gp(const WorldDev &W, int lps);
 cudaError_t launch_step(const WorldDev &W, const LaunchCfg &cfg, int n_steps, cudaStream_t st);
 cudaError_t launch_advance(long long *d_step, int n, cudaStream_t st);
 cudaError_t launch_init(const WorldDev &W, const float *d_origin, const float *d_quat,

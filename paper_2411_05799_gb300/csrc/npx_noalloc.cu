@@ -57,7 +57,8 @@ extern "C" int npx_step_noalloc(const npx_device_world *d, int n_steps, void *st
                  "(the size of its static scratch array)", d->n_scenes, NOALLOC_MAX_SCENES);
         return noalloc_fail(NPX_ERANGE, buf);
     }
-    const int lps = d->lanes_per_scene, wpb = d->warps_per_block;
+    const int lps = d->lanes_per_scene;
+    int wpb = d->warps_per_block;
     if (lps != 4 && lps != 8 && lps != 16 && lps != 32)
         return noalloc_fail(NPX_EINVAL, "npx_step_noalloc: lanes_per_scene must be 4, 8, 16 or 32");
     if (wpb < 1 || wpb > 16) return noalloc_fail(NPX_EINVAL, "npx_step_noalloc: warps_per_block must be 1..16");
@@ -129,7 +130,9 @@ extern "C" int npx_step_noalloc(const npx_device_world *d, int n_steps, void *st
     W.order = reinterpret_cast<const int *>(scratch + NOALLOC_HEADER_WORDS);
     W.n_sched = W.S;
 
-    int nb = npx::step_blocks_per_sm(W, lps, wpb, &e);   // also raises the kernel's smem limit
+    int nb = npx::step_blocks_per_sm(W, lps, wpb, 0, &e);   // also raises the kernel's smem limit
+    if (nb < 1 && npx::step_fits_bare(W, lps, wpb))         // (see clamp_cfg_for)
+        while (nb < 1 && wpb > 1 && e == cudaSuccess) nb = npx::step_blocks_per_sm(W, lps, --wpb, 0, &e);
     if (e != cudaSuccess || nb < 1)
         return noalloc_fail(NPX_ERANGE, "npx_step_noalloc: this launch shape does not fit on an SM");
     int n_sm = 0;

@@ -68,6 +68,35 @@ __device__ __forceinline__ uint32_t gor(uint32_t v) {
 
 // ------------------------------------------------------------------------ small linear algebra
 
+// Sums of products with their rounding written out, for the step loop of the flat build without
+// options (PIN): which product of a x + b y is fused (the first, or with SECOND the second) is
+// otherwise the compiler's choice, it moves with the code around it, and the friction solve's
+// moments cancel, so it shows in the result.  Without PIN they are the plain expressions.
+template <bool PIN, bool SECOND = false>
+__device__ __forceinline__ float pin2(float a, float x, float b, float y) {
+    if constexpr (PIN) return SECOND ? fmaf(b, y, __fmul_rn(a, x)) : fmaf(a, x, __fmul_rn(b, y));
+    return a * x + b * y;
+}
+template <bool PIN>   // a x - b y
+__device__ __forceinline__ float pind(float a, float x, float b, float y) {
+    if constexpr (PIN) return fmaf(a, x, -__fmul_rn(b, y));
+    return a * x - b * y;
+}
+template <bool PIN, bool SECOND = false>
+__device__ __forceinline__ float pin3(float a, float x, float b, float y, float c, float z) {
+    if constexpr (PIN) return fmaf(c, z, pin2<PIN, SECOND>(a, x, b, y));
+    return a * x + b * y + c * z;
+}
+template <bool PIN, bool SECOND = false>
+__device__ __forceinline__ float pin3(const float a[3], const float x[3]) {
+    return pin3<PIN, SECOND>(a[0], x[0], a[1], x[1], a[2], x[2]);
+}
+template <bool PIN>   // a + x y
+__device__ __forceinline__ float pinf(float x, float y, float a) {
+    if constexpr (PIN) return fmaf(x, y, a);
+    return a + x * y;
+}
+
 struct Sym {  // symmetric 3x3
     float xx, yy, zz, xy, xz, yz;
 };
@@ -122,6 +151,27 @@ __device__ __forceinline__ void world_sym(const float R[9], const Sym &S, const 
     mat_vec(R, b, y);
 }
 
+template <bool PIN>
+__device__ __forceinline__ void mat_vec_pin(const float R[9], const float x[3], float y[3]) {
+    y[0] = pin3<PIN>(R, x);
+    y[1] = pin3<PIN>(R + 3, x);
+    y[2] = pin3<PIN>(R + 6, x);
+}
+template <bool PIN>
+__device__ __forceinline__ void sym_mul_pin(const Sym &a, const float x[3], float y[3]) {
+    y[0] = pin3<PIN>(a.xx, x[0], a.xy, x[1], a.xz, x[2]);
+    y[1] = pin3<PIN>(a.xy, x[0], a.yy, x[1], a.yz, x[2]);
+    y[2] = pin3<PIN>(a.xz, x[0], a.yz, x[1], a.zz, x[2]);
+}
+template <bool PIN>
+__device__ __forceinline__ void world_sym_pin(const float R[9], const Sym &S, const float x[3], float y[3]) {
+    const float a[3] = {pin3<PIN>(R[0], x[0], R[3], x[1], R[6], x[2]), pin3<PIN>(R[1], x[0], R[4], x[1], R[7], x[2]),
+                        pin3<PIN>(R[2], x[0], R[5], x[1], R[8], x[2])};
+    float b[3];
+    sym_mul_pin<PIN>(S, a, b);
+    mat_vec_pin<PIN>(R, b, y);
+}
+
 __device__ __forceinline__ void quat_mul(const float a[4], const float b[4], float c[4]) {
     float t0 = a[0] * b[0] - a[1] * b[1] - a[2] * b[2] - a[3] * b[3];
     float t1 = a[0] * b[1] + a[1] * b[0] + a[2] * b[3] - a[3] * b[2];
@@ -135,12 +185,12 @@ __device__ __forceinline__ void quat_mul(const float a[4], const float b[4], flo
 // 1e-12); outside it the library functions are used.  Per-step rotation increments and friction
 // corrections are almost always tiny, so this removes the range reduction from the hot path.
 // (returned by value: a pointer into the caller would force its results into local memory)
-__device__ __noinline__ float2 sincos_large(float x) {
+static __device__ __noinline__ float2 sincos_large(float x) {
     float s, c;
     sincosf(x, &s, &c);
     return make_float2(s, c);
 }
-__device__ __noinline__ float asin_large(float x) { return asinf(x); }
+static __device__ __noinline__ float asin_large(float x) { return asinf(x); }
 
 __device__ __forceinline__ void sincos_poly(float x, float *s, float *c) {   // |x| <= 1/16
     const float x2 = x * x;
@@ -172,8 +222,8 @@ __device__ __forceinline__ float asin_small(float x) {
 __host__ __device__ inline int tiles_offset(int max_points, int max_links) {
     return (16 * max_points + 58 * max_links + 15) & ~15;
 }
-// (16 bytes after the boxes: at shape updates their area holds the points' links, shifted by up to
-// 3 bytes)
+// 16 spare bytes after the boxes: at shape updates their area holds the points' links, shifted by up
+// to 3 bytes
 __host__ __device__ inline int slot_bytes(int max_points, int max_links, int lps) {
     return tiles_offset(max_points, max_links) + 32 * ((max_points + lps - 1) / lps) + 16;
 }
@@ -391,7 +441,8 @@ struct Shape {
 // the mass moments about it, then the CoG, the inertia about the CoG (parallel-axis theorem; gref
 // is close to the CoG, so the FP32 sums do not cancel) and a recentring of the stored offsets.
 // Being a function of theta alone, the result does not depend on where a launch (chunk) starts.
-template <int LPS>
+// GP: the offsets go to global memory (pts), and the construction positions are read where they are.
+template <int LPS, bool GP>
 __device__ __noinline__ void shape_update(const WorldDev &W, int s, int p0, int np, int l0, int nl,
                                           const float *th, float *fr, float4 *pts, int gl,
                                           Shape &sh) {
@@ -401,10 +452,14 @@ __device__ __noinline__ void shape_update(const WorldDev &W, int s, int p0, int 
     // (as whole aligned words where their address allows, the ends byte by byte; every read stays
     // inside the scene's bytes, and nothing waits for a load before the frames are done)
     const uint8_t *src = W.plink + p0;
-    uint8_t *lk = reinterpret_cast<uint8_t *>(pts) + tiles_offset(W.max_points, W.max_links) +
+    // (a slot without its points starts with the frames)
+    uint8_t *lk = (GP ? reinterpret_cast<uint8_t *>(fr) + tiles_offset(0, W.max_links)
+                      : reinterpret_cast<uint8_t *>(pts) + tiles_offset(W.max_points, W.max_links)) +
                   ((uint32_t)(uintptr_t)src & 3u);
+    if constexpr (!GP) {
 #pragma unroll 8
-    for (int i = gl; i < np; i += LPS) cp_async16(pts + i, W.p0m + p0 + i);
+        for (int i = gl; i < np; i += LPS) cp_async16(pts + i, W.p0m + p0 + i);
+    }
     const int h = min((int)((4u - ((uint32_t)(uintptr_t)src & 3u)) & 3u), np);
     const int nw = (np - h) >> 2, e = h + 4 * nw + gl;
     uint8_t head = 0, tail = 0;
@@ -421,7 +476,7 @@ __device__ __noinline__ void shape_update(const WorldDev &W, int s, int p0, int 
     float a[10] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
     for (int i = gl; i < np; i += LPS) {
-        const float4 q = pts[i];
+        const float4 q = GP ? W.p0m[p0 + i] : pts[i];
         float p[3];
         fk_point(fr, q, lk[i], p);
         const float dx = p[0] - gref[0], dy = p[1] - gref[1], dz = p[2] - gref[2], m = q.w;
@@ -514,7 +569,7 @@ __device__ __forceinline__ void scache_store(const WorldDev &W, int s, int np, c
 // Reads the posed shape of scene s (-1: no scene) from its cache entry into the slot: the offsets,
 // the mass properties and, when they were written with this many lanes per scene on every scene
 // of the warp, the tile boxes (else they are rebuilt from the offsets).  Returns rmax.
-template <int LPS>
+template <int LPS, bool GP>
 __device__ __forceinline__ float scache_load(const WorldDev &W, int s, int np, float4 *pts, float4 *tb, Shape &sh,
                                              int gl) {
     const float4 *e = W.scache + (size_t)(s < 0 ? 0 : s) * scache_stride(W.scache_mp, W.scache_mt, W.scache_ml);
@@ -526,7 +581,10 @@ __device__ __forceinline__ float scache_load(const WorldDev &W, int s, int np, f
     if (s >= 0) { m0 = m[0]; m1 = m[1]; m2 = m[2]; m3 = m[3]; m4 = m[4]; }
     const bool tb_ok = __all_sync(FULL_MASK, __float_as_int(m4.y) == LPS);
 #pragma unroll 4
-    for (int i = gl; i < np; i += LPS) cp_async16(pts + i, e + i);
+    for (int i = gl; i < np; i += LPS) {
+        if constexpr (GP) pts[i] = e[i];
+        else cp_async16(pts + i, e + i);
+    }
     if (tb_ok)
         for (int i = gl; i < 2 * nt; i += LPS) cp_async16(tb + i, e + W.scache_mp + i);
     cp_async_wait_all();
@@ -636,7 +694,7 @@ constexpr float GP_STEP = 0.087266462599716478846f;   // 5 degrees
 // +-GP_KMAX; motors the scene lacks are ignored), 010 acc = foot-contact bit x of the last step,
 // 011 acc = x, 100 jump to x if acc != 0, 101 acc = ~acc, 110 inc, 111 dec (8-bit accumulator,
 // the program counter wraps after address 31).
-__device__ __noinline__ void gp_run(const WorldDev &W, int s, int j0, int nj, uint32_t sensors) {
+static __device__ __noinline__ void gp_run(const WorldDev &W, int s, int j0, int nj, uint32_t sensors) {
     const uint8_t *prog = W.gp_prog + (size_t)GP_LEN * s;
     int8_t *k = W.gp_k + j0;
     uint32_t p = W.gp_pc[s] & (GP_LEN - 1), a = W.gp_acc[s];
@@ -1160,8 +1218,9 @@ __device__ __forceinline__ void arena_wrench(const WorldDev &W, unsigned char *x
 
 // OPT: the friction-model options (W.fric_mode) are compiled in; without them the step is the
 // least squares of Eqs. 1-6 as written, with no test of the options in the step loop; ARENA:
-// robot-robot contact within arenas (below)
-template <int LPS, bool FLAT, bool OPT, bool ARENA>
+// robot-robot contact within arenas (below); GP: the posed offsets pts lie in global memory, where
+// they stay in L1 and L2, instead of the slot
+template <int LPS, bool FLAT, bool OPT, bool ARENA, bool GP>
 __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *fr, float *th,
                           float *th_old, float4 *tb, int n_steps, long long step0, unsigned char *xch,
                           int sbytes, const CUtensorMap *tmap, int item) {
@@ -1204,9 +1263,9 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
     // the posed shape of the current joint angles: read from the posed-shape cache when the
     // launch says every entry is current, else rebuilt (and written to the cache when there is one)
     if (!ARENA && W.scache_mode == 2) {
-        rmax = scache_load<LPS>(W, valid ? s : -1, np, pts, tb, sh, gl);
+        rmax = scache_load<LPS, GP>(W, valid ? s : -1, np, pts, tb, sh, gl);
     } else {
-        shape_update<LPS>(W, valid ? s : 0, p0, np, l0, nl, th, fr, pts, gl, sh);
+        shape_update<LPS, GP>(W, valid ? s : 0, p0, np, l0, nl, th, fr, pts, gl, sh);
         rmax = tile_bounds<LPS>(pts, np, tb, gl);
         if (!ARENA && W.scache_mode != 0 && valid) scache_store<LPS>(W, s, np, pts, tb, sh, rmax, fr, l0, nl, gl);
     }
@@ -1264,6 +1323,7 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
     // the normal forces; the friction impulse's torque about the horizontal axes
     const bool weighted = OPT && (W.fric_mode & 1) != 0, tilt = OPT && (W.fric_mode & 2) != 0;
     float iM = 1.0f / shr.M;
+    constexpr bool PIN = FLAT && !OPT && !ARENA;
     const bool actuated = W.act_mode != 0;
     // Candidate tiles: those whose box came within CULL_MARGIN of the highest ground at the last
     // cull.  slack is the height above the highest ground of the lowest box left out then, minus
@@ -1312,7 +1372,7 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
                 }
             }
             __syncwarp();
-            shape_update<LPS>(W, valid ? s : 0, p0, np, l0, nl, th, fr, pts, gl, sh);
+            shape_update<LPS, GP>(W, valid ? s : 0, p0, np, l0, nl, th, fr, pts, gl, sh);
             rmax = tile_bounds<LPS>(pts, np, tb, gl);
             if (!ARENA && W.scache_mode != 0 && valid) scache_store<LPS>(W, s, np, pts, tb, sh, rmax, fr, l0, nl, gl);
             shr = sh;
@@ -1326,7 +1386,7 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
         }
 
         float om[3];
-        world_sym(R, shr.Ii, L, om);
+        world_sym_pin<PIN>(R, shr.Ii, L, om);
 
         // -- (arenas) contact forces and their torques about the CoG from the other robots
         float rf[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -1418,7 +1478,7 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
             if (kf < 64) {
                 const float4 lo = tb[2 * kf], hi = tb[2 * kf + 1];
                 const float mid[3] = {0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z)};
-                mat_vec(R, mid, o);
+                mat_vec_pin<PIN>(R, mid, o);
             }
         } else {
             if (__any_sync(FULL_MASK, ref_stale)) {
@@ -1456,9 +1516,9 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
                 const int ia = gl + (ja + 32 * hw) * LPS, ib = gl + (jb + 32 * hw) * LPS;
                 const bool oka = ia < np, okb = two && ib < np;
                 const float4 pa = pts[oka ? ia : 0], pb = pts[okb ? ib : 0];
-                const float rxa = R[0] * pa.x + R[1] * pa.y + R[2] * pa.z, rxb = R[0] * pb.x + R[1] * pb.y + R[2] * pb.z;
-                const float rya = R[3] * pa.x + R[4] * pa.y + R[5] * pa.z, ryb = R[3] * pb.x + R[4] * pb.y + R[5] * pb.z;
-                const float rza = R[6] * pa.x + R[7] * pa.y + R[8] * pa.z, rzb = R[6] * pb.x + R[7] * pb.y + R[8] * pb.z;
+                const float rxa = pin3<PIN>(R[0], pa.x, R[1], pa.y, R[2], pa.z), rxb = pin3<PIN>(R[0], pb.x, R[1], pb.y, R[2], pb.z);
+                const float rya = pin3<PIN>(R[3], pa.x, R[4], pa.y, R[5], pa.z), ryb = pin3<PIN>(R[3], pb.x, R[4], pb.y, R[5], pb.z);
+                const float rza = pin3<PIN>(R[6], pa.x, R[7], pa.y, R[8], pa.z), rzb = pin3<PIN>(R[6], pb.x, R[7], pb.y, R[8], pb.z);
                 const float za = c[2] + rza, zb = c[2] + rzb;
                 const float ha = ground_win<FLAT>(W, hm, win + wsh, wx0, wy0, c[0] + rxa, c[1] + rya);
                 const float hb = ground_win<FLAT>(W, hm, win + wsh, wx0, wy0, c[0] + rxb, c[1] + ryb);
@@ -1468,12 +1528,12 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
                 // step after, 9.78 before.  On flat ground most tiles touch and the branch costs more
                 // than it skips (2.17 -> 2.49 ms a second of 4,096 hexapods), so it is not taken.
                 if (FLAT || ca || cb) {
-                    const float vza = v[2] + (om[0] * rya - om[1] * rxa), vzb = v[2] + (om[0] * ryb - om[1] * rxb);
-                    const float Fa = ca ? fmaxf(0.f, pa.w * (kw2 * (ha - za) - kc * vza)) : 0.f;
-                    const float Fb = cb ? fmaxf(0.f, pb.w * (kw2 * (hb - zb) - kc * vzb)) : 0.f;
+                    const float vza = v[2] + pind<PIN>(om[0], rya, om[1], rxa), vzb = v[2] + pind<PIN>(om[0], ryb, om[1], rxb);
+                    const float Fa = ca ? fmaxf(0.f, pa.w * pind<PIN>(kw2, ha - za, kc, vza)) : 0.f;
+                    const float Fb = cb ? fmaxf(0.f, pb.w * pind<PIN>(kw2, hb - zb, kc, vzb)) : 0.f;
                     knw[hw] |= (ca ? 1u << ja : 0u) | (cb ? 1u << jb : 0u);
-                    acc[0] += Fa; acc[1] += rya * Fa; acc[2] -= rxa * Fa;
-                    acc[0] += Fb; acc[1] += ryb * Fb; acc[2] -= rxb * Fb;
+                    acc[0] += Fa; acc[1] = pinf<PIN>(rya, Fa, acc[1]); acc[2] = PIN ? fmaf(-rxa, Fa, acc[2]) : acc[2] - rxa * Fa;
+                    acc[0] += Fb; acc[1] = pinf<PIN>(ryb, Fb, acc[1]); acc[2] = PIN ? fmaf(-rxb, Fb, acc[2]) : acc[2] - rxb * Fb;
                     // friction set C: in contact now and last step; a row's weight is 1, or its normal
                     // force with force-weighted friction.  Sums: weight, weight x d, weight x d d^T
                     const float wa = (ca && ((kp >> ja) & 1u)) ? (weighted ? Fa : 1.f) : 0.f;
@@ -1485,10 +1545,10 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
                     acc[3] += wa; acc[3] += wb;
                     acc[4] += a0; acc[5] += a1; acc[6] += a2;
                     acc[4] += b0; acc[5] += b1; acc[6] += b2;
-                    acc[7] += a0 * da0; acc[8] += a1 * da1; acc[9] += a2 * da2;
-                    acc[10] += a0 * da1; acc[11] += a0 * da2; acc[12] += a1 * da2;
-                    acc[7] += b0 * db0; acc[8] += b1 * db1; acc[9] += b2 * db2;
-                    acc[10] += b0 * db1; acc[11] += b0 * db2; acc[12] += b1 * db2;
+                    acc[7] = pinf<PIN>(a0, da0, acc[7]); acc[8] = pinf<PIN>(a1, da1, acc[8]); acc[9] = pinf<PIN>(a2, da2, acc[9]);
+                    acc[10] = pinf<PIN>(a0, da1, acc[10]); acc[11] = pinf<PIN>(a0, da2, acc[11]); acc[12] = pinf<PIN>(a1, da2, acc[12]);
+                    acc[7] = pinf<PIN>(b0, db0, acc[7]); acc[8] = pinf<PIN>(b1, db1, acc[8]); acc[9] = pinf<PIN>(b2, db2, acc[9]);
+                    acc[10] = pinf<PIN>(b0, db1, acc[10]); acc[11] = pinf<PIN>(b0, db2, acc[11]); acc[12] = pinf<PIN>(b1, db2, acc[12]);
                 }
             }
         }
@@ -1499,9 +1559,13 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
         const float nC = acc[3];
         const float in = nC > 0.f ? __fdividef(1.f, nC) : 0.f;
         const float e0 = acc[4] * in, e1 = acc[5] * in, e2 = acc[6] * in;   // centroid - o
-        const float gb[3] = {o[0] + e0, o[1] + e1, o[2] + e2};
-        const Sym M2 = {acc[7] - nC * (e0 * e0), acc[8] - nC * (e1 * e1), acc[9] - nC * (e2 * e2),
-                        acc[10] - nC * (e0 * e1), acc[11] - nC * (e0 * e2), acc[12] - nC * (e1 * e2)};
+        const float gb[3] = {PIN ? __fadd_rn(o[0], e0) : o[0] + e0, PIN ? __fadd_rn(o[1], e1) : o[1] + e1,
+                             PIN ? __fadd_rn(o[2], e2) : o[2] + e2};
+        const Sym M2 = PIN ? Sym{fmaf(-nC, __fmul_rn(e0, e0), acc[7]), fmaf(-nC, __fmul_rn(e1, e1), acc[8]),
+                                 fmaf(-nC, __fmul_rn(e2, e2), acc[9]), fmaf(-nC, __fmul_rn(e0, e1), acc[10]),
+                                 fmaf(-nC, __fmul_rn(e0, e2), acc[11]), fmaf(-nC, __fmul_rn(e1, e2), acc[12])}
+                           : Sym{acc[7] - nC * (e0 * e0), acc[8] - nC * (e1 * e1), acc[9] - nC * (e2 * e2),
+                                 acc[10] - nC * (e0 * e1), acc[11] - nC * (e0 * e2), acc[12] - nC * (e1 * e2)};
 
         // -- semi-implicit Euler
         float vs[3], Ls[3], cs[3], qs[4], oms[3];
@@ -1515,7 +1579,7 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
             vs[0] += dt * (rf[0] * iM); vs[1] += dt * (rf[1] * iM); vs[2] += dt * (rf[2] * iM);
             Ls[0] += dt * rf[3]; Ls[1] += dt * rf[4]; Ls[2] += dt * rf[5];
         }
-        world_sym(R, shr.Ii, Ls, oms);
+        world_sym_pin<PIN>(R, shr.Ii, Ls, oms);
         cs[0] = c[0] + dt * vs[0]; cs[1] = c[1] + dt * vs[1]; cs[2] = c[2] + dt * vs[2];
         // rotation increment dR = exp([u]x), u = dt w*: q* = dq (x) q and R* = dR R, so a point's
         // offset moves from rho to (1 + D) rho with D = dR - 1 = a [u]x + b [u]x^2
@@ -1525,7 +1589,7 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
                            // friction-set centroid above the integrated CoG: [(1 + D) gb]_z
         {
             const float px = dt * oms[0], py = dt * oms[1], pz = dt * oms[2];
-            const float a2 = px * px + py * py + pz * pz;
+            const float a2 = pin3<PIN>(px, px, py, py, pz, pz);
             const float ra = a2 > 0.f ? rsqrtf(a2) : 0.f;   // 1 / |u|
             const float a = a2 * ra;
             float dq[4] = {1.f, 0.f, 0.f, 0.f};
@@ -1542,10 +1606,28 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
                 rzc = gb[2] + (-fa * py + fb * pz * px) * gb[0] + (fa * px + fb * pz * py) * gb[1] +
                       fb * (pz * pz - a2) * gb[2];
             // [u]x^2 = u u^T - |u|^2 1
-            Dm[0] = fb * (px * px - a2); Dm[1] = -fa * pz + fb * px * py; Dm[2] = fa * py + fb * px * pz;
-            Dm[3] = fa * pz + fb * py * px; Dm[4] = fb * (py * py - a2); Dm[5] = -fa * px + fb * py * pz;
-            quat_mul(dq, q, qs);
-            const float inv = rsqrtf(qs[0] * qs[0] + qs[1] * qs[1] + qs[2] * qs[2] + qs[3] * qs[3]);
+            float qn2;
+            if constexpr (PIN) {
+                const float fx = __fmul_rn(fb, px), fy = __fmul_rn(fb, py);
+                Dm[0] = __fmul_rn(fb, fmaf(px, px, -a2));
+                Dm[1] = fmaf(fx, py, -__fmul_rn(fa, pz));
+                Dm[2] = fmaf(fa, py, __fmul_rn(fx, pz));
+                Dm[3] = fmaf(fy, px, __fmul_rn(fa, pz));
+                Dm[4] = __fmul_rn(fb, fmaf(py, py, -a2));
+                Dm[5] = fmaf(fy, pz, -__fmul_rn(fa, px));
+                // q* = dq (x) q
+                qs[0] = fmaf(-dq[3], q[3], fmaf(-dq[2], q[2], pind<true>(dq[0], q[0], dq[1], q[1])));
+                qs[1] = fmaf(-dq[3], q[2], fmaf(dq[2], q[3], pin2<true>(dq[0], q[1], dq[1], q[0])));
+                qs[2] = fmaf(dq[3], q[1], fmaf(dq[2], q[0], pind<true>(dq[0], q[2], dq[1], q[3])));
+                qs[3] = fmaf(dq[3], q[0], fmaf(-dq[2], q[1], pin2<true>(dq[0], q[3], dq[1], q[2])));
+                qn2 = fmaf(qs[3], qs[3], pin3<true>(qs, qs));
+            } else {
+                Dm[0] = fb * (px * px - a2); Dm[1] = -fa * pz + fb * px * py; Dm[2] = fa * py + fb * px * pz;
+                Dm[3] = fa * pz + fb * py * px; Dm[4] = fb * (py * py - a2); Dm[5] = -fa * px + fb * py * pz;
+                quat_mul(dq, q, qs);
+                qn2 = qs[0] * qs[0] + qs[1] * qs[1] + qs[2] * qs[2] + qs[3] * qs[3];
+            }
+            const float inv = rsqrtf(qn2);
             qs[0] *= inv; qs[1] *= inv; qs[2] *= inv; qs[3] *= inv;
             // largest downward move of any point this step: dt max(0, -v*_z) from the CoG plus the
             // rotation's: for x = R r, ((dR - 1) x)_z = sin|u| (n x x)_z + (1 - cos|u|) (n (n.x) - x)_z
@@ -1576,13 +1658,13 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
                 float po[3];
                 fk_point_words(fr, a0, W.plink[p0 + i], po);
                 const float4 ro = make_float4(po[0] - gold[0], po[1] - gold[1], po[2] - gold[2], 0.f);
-                const float rx = R[0] * r.x + R[1] * r.y + R[2] * r.z;
-                const float ry = R[3] * r.x + R[4] * r.y + R[5] * r.z;
+                const float rx = pin3<PIN>(R[0], r.x, R[1], r.y, R[2], r.z);
+                const float ry = pin3<PIN>(R[3], r.x, R[4], r.y, R[5], r.z);
                 const float ux = rx - gb[0];
                 const float uy = ry - gb[1];
                 const float d[3] = {ro.x - r.x, ro.y - r.y, ro.z - r.z};
-                const float kx = R[0] * d[0] + R[1] * d[1] + R[2] * d[2];
-                const float ky = R[3] * d[0] + R[4] * d[1] + R[5] * d[2];
+                const float kx = pin3<PIN>(R, d);
+                const float ky = pin3<PIN>(R + 3, d);
                 float wk = 1.f;   // the row's weight: its normal force this step (as in pass 1)
                 if (weighted) {
                     const float rz = R[6] * r.x + R[7] * r.y + R[8] * r.z;
@@ -1592,40 +1674,42 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
                     wk = fmaxf(0.f, r.w * (kw2 * (h - z) - kc * vz));
                 }
                 const float wux = wk * ux, wuy = wk * uy;
-                f6[0] += wux; f6[1] += wuy; f6[2] += wux * ux + wuy * uy;
-                f6[3] += wk * kx; f6[4] += wk * ky; f6[5] += wux * ky - wuy * kx;
+                f6[0] += wux; f6[1] += wuy; f6[2] += pin2<PIN>(wux, ux, wuy, uy);
+                f6[3] += wk * kx; f6[4] += wk * ky; f6[5] += pind<PIN>(wux, ky, wuy, kx);
             }
             gsum<LPS, 6>(f6);
         }
         if (nC > 0.f) {
             const float ax[3] = {1.f + Dm[0], Dm[1], Dm[2]}, ay[3] = {Dm[3], 1.f + Dm[4], Dm[5]};
             const float bx[3] = {Dm[0], Dm[1], Dm[2]}, by[3] = {Dm[3], Dm[4], Dm[5]};
-            float Max[3], May[3];
-            sym_mul(M2, ax, Max);
-            sym_mul(M2, ay, May);
-            const float S2 = ax[0] * Max[0] + ax[1] * Max[1] + ax[2] * Max[2] +
-                             ay[0] * May[0] + ay[1] * May[1] + ay[2] * May[2];
-            const float X = -((Max[0] * by[0] + Max[1] * by[1] + Max[2] * by[2]) -
-                              (May[0] * bx[0] + May[1] * bx[1] + May[2] * bx[2]));
-            const float sbx = ax[0] * gb[0] + ax[1] * gb[1] + ax[2] * gb[2];  // source centroid - c*
-            const float sby = ay[0] * gb[0] + ay[1] * gb[1] + ay[2] * gb[2];
-            const float tDx = -dt * vs[0] - (bx[0] * gb[0] + bx[1] * gb[1] + bx[2] * gb[2]);
-            const float tDy = -dt * vs[1] - (by[0] * gb[0] + by[1] * gb[1] + by[2] * gb[2]);
+            const float m0[3] = {M2.xx, M2.xy, M2.xz}, m1[3] = {M2.xy, M2.yy, M2.yz}, m2[3] = {M2.xz, M2.yz, M2.zz};
+            const float Max[3] = {pin3<PIN>(m0, ax), pin3<PIN>(m1, ax), pin3<PIN>(m2, ax)};
+            const float May[3] = {pin3<PIN, true>(m0, ay), pin3<PIN, true>(m1, ay), pin3<PIN, true>(m2, ay)};
+            const float S2 = PIN ? fmaf(ay[2], May[2], fmaf(ay[1], May[1], fmaf(ay[0], May[0], pin3<PIN>(ax, Max))))
+                                 : ax[0] * Max[0] + ax[1] * Max[1] + ax[2] * Max[2] +
+                                   ay[0] * May[0] + ay[1] * May[1] + ay[2] * May[2];
+            const float X = -(pin3<PIN>(Max, by) - pin3<PIN>(May, bx));
+            const float sbx = pin3<PIN>(ax, gb);  // source centroid - c*
+            const float sby = pin3<PIN, true>(ay, gb);
+            const float tDx = PIN ? fmaf(-dt, vs[0], -pin3<PIN>(bx, gb)) : -dt * vs[0] - pin3<PIN>(bx, gb);
+            const float tDy = PIN ? fmaf(-dt, vs[1], -pin3<PIN, true>(by, gb)) : -dt * vs[1] - pin3<PIN>(by, gb);
             // a rotation needs two distinct points (force-weighted: a weighted mean spread about
             // the centre of pressure above 1e-6 m^2, far above the rounding left by the moments'
             // cancellation when the weight sits on one point)
             float a3 = (weighted ? S2 > 1e-6f * nC : (nC >= 2.f && S2 > 1e-12f)) ? __fdividef(X, S2) : 0.f;
             a3 = fminf(fmaxf(a3, -1.f), 1.f);
-            const float t1 = fmaxf(0.f, 1.f - a3 * a3);
+            const float t1 = fmaxf(0.f, PIN ? fmaf(-a3, a3, 1.f) : 1.f - a3 * a3);
             const float cD = t1 > 0.f ? t1 * rsqrtf(t1) : 0.f;       // cos(alpha_D)
             const float r1 = __fdividef(1.f, 1.f + cD);
             const float cm1 = -a3 * a3 * r1;                          // cos(alpha_D) - 1
             const float dDx = -sbx, dDy = -sby;                       // CoG minus centroid
-            const float DDx = tDx + cm1 * dDx - a3 * dDy;             // uncapped CoG shift
-            const float DDy = tDy + a3 * dDx + cm1 * dDy;
+            // uncapped CoG shift
+            const float DDx = PIN ? fmaf(-a3, dDy, fmaf(cm1, dDx, tDx)) : tDx + cm1 * dDx - a3 * dDy;
+            const float DDy = PIN ? fmaf(cm1, dDy, fmaf(a3, dDx, tDy)) : tDy + a3 * dDx + cm1 * dDy;
             // maximum static friction (Coulomb cap on the impulse that undoes the slip)
             const float sh2 = 0.5f * a3 * a3 * r1;                    // sin^2(alpha_D / 2)
-            const float u2 = tDx * tDx + tDy * tDy + 4.f * sh2 * S2 * in;
+            const float u2 = PIN ? fmaf(4.f * sh2 * S2, in, pin2<PIN>(tDx, tDx, tDy, tDy))
+                                 : tDx * tDx + tDy * tDy + 4.f * sh2 * S2 * in;
             const float Jreq = shr.M * (u2 > 0.f ? u2 * rsqrtf(u2) : 0.f) * idt;
             const float Jmax = mu * dt * FN;
             const float sc = (Jreq <= Jmax) ? 1.f : __fdividef(Jmax, Jreq);
@@ -1638,8 +1722,8 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
             if (!OPT && fabsf(a3) <= 0.0625f) sincos_poly(0.5f * sc * aD, &s1, &c1);
             else sincos_small(0.5f * sc * aD, &s1, &c1);
             const float sin1 = 2.f * s1 * c1, cm1s = -2.f * s1 * s1;
-            float dx1 = sc * tDx + cm1s * dDx - sin1 * dDy;
-            float dy1 = sc * tDy + sin1 * dDx + cm1s * dDy;
+            float dx1 = PIN ? fmaf(-sin1, dDy, pin2<PIN>(sc, tDx, cm1s, dDx)) : sc * tDx + cm1s * dDx - sin1 * dDy;
+            float dy1 = PIN ? fmaf(cm1s, dDy, pin2<PIN>(sc, tDy, sin1, dDx)) : sc * tDy + sin1 * dDx + cm1s * dDy;
             float A = sc * aD;
             if (tick) {
                 const float kbx = f6[0] * in, kby = f6[1] * in;
@@ -1661,8 +1745,8 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
             }
             cn[0] = cs[0] + dx1;
             cn[1] = cs[1] + dy1;
-            vn[0] = vs[0] + sc * DDx * idt;
-            vn[1] = vs[1] + sc * DDy * idt;
+            vn[0] = pinf<PIN>(sc * DDx, idt, vs[0]);
+            vn[1] = pinf<PIN>(sc * DDy, idt, vs[1]);
             // angular momentum of the yaw correction: (sc alpha_D / dt) R* Ib R*^T z
             float Rs[9];
             quat_mat(qs, Rs);
@@ -1673,11 +1757,11 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
             } else {
                 const float ez[3] = {Rs[6], Rs[7], Rs[8]};   // R*^T z
                 float bz[3];
-                sym_mul(shr.Ib, ez, bz);
-                mat_vec(Rs, bz, Iz);
+                sym_mul_pin<PIN>(shr.Ib, ez, bz);
+                mat_vec_pin<PIN>(Rs, bz, Iz);
             }
             const float w = sc * aD * idt;
-            Ln[0] = Ls[0] + w * Iz[0]; Ln[1] = Ls[1] + w * Iz[1]; Ln[2] = Ls[2] + w * Iz[2];
+            Ln[0] = pinf<PIN>(w, Iz[0], Ls[0]); Ln[1] = pinf<PIN>(w, Iz[1], Ls[1]); Ln[2] = pinf<PIN>(w, Iz[2], Ls[2]);
             if (tilt) {
                 // the friction impulse J = M (v_new - v*) acts at the friction-set centroid,
                 // rzc below the CoG: the x and y components of its moment r x J
@@ -1687,8 +1771,15 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
             }
             float sa = s1, ca = c1;   // A is the capped dynamic angle, unless the joints moved
             if (OPT || tick) sincos_small(0.5f * A, &sa, &ca);
-            const float qz[4] = {ca, 0.f, 0.f, sa};
-            quat_mul(qz, qs, qn);
+            if constexpr (PIN) {   // (ca, 0, 0, sa) (x) q*
+                qn[0] = fmaf(-sa, qs[3], __fmul_rn(ca, qs[0]));
+                qn[1] = fmaf(-sa, qs[2], __fmul_rn(ca, qs[1]));
+                qn[2] = fmaf(sa, qs[1], __fmul_rn(ca, qs[2]));
+                qn[3] = fmaf(sa, qs[0], __fmul_rn(ca, qs[3]));
+            } else {
+                const float qz[4] = {ca, 0.f, 0.f, sa};
+                quat_mul(qz, qs, qn);
+            }
         }
 
         // -- freeze a scene whose state is no longer finite or has left any sane range
@@ -1750,7 +1841,7 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
     __syncwarp();
 }
 
-template <int LPS, bool FLAT, bool OPT, bool ARENA>
+template <int LPS, bool FLAT, bool OPT, bool ARENA, bool GP>
 __device__ __forceinline__ void step_body(const WorldDev &W, int n_steps, int sbytes, const CUtensorMap *tmap) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // (height maps) a 128-byte aligned base, so that every window is aligned for its TMA box
@@ -1761,11 +1852,13 @@ __device__ __forceinline__ void step_body(const WorldDev &W, int n_steps, int sb
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane / LPS, gl = lane % LPS;
     unsigned char *slot = smem + (size_t)(warp * G + g) * sbytes;
-    float4 *pts = reinterpret_cast<float4 *>(slot);
-    float *fr = reinterpret_cast<float *>(slot + 16 * W.max_points);
+    const int sp = GP ? 0 : W.max_points;   // points in the slot
+    float4 *pts = GP ? W.pscr + ((size_t)(blockIdx.x * (blockDim.x / 32) + warp) * G + g) * W.max_points
+                     : reinterpret_cast<float4 *>(slot);
+    float *fr = reinterpret_cast<float *>(slot + 16 * sp);
     float *th = fr + 12 * W.max_links;
     float *th_old = th + W.max_links;
-    float4 *tb = reinterpret_cast<float4 *>(slot + tiles_offset(W.max_points, W.max_links));
+    float4 *tb = reinterpret_cast<float4 *>(slot + tiles_offset(sp, W.max_links));
     // (arenas) the scene's exchange area, after all slots of the block
     unsigned char *xch = smem + (size_t)(blockDim.x / 32) * G * sbytes + (size_t)(warp * G + g) * xch_bytes(W.max_chunks);
     const long long step0 = *W.step;
@@ -1778,15 +1871,17 @@ __device__ __forceinline__ void step_body(const WorldDev &W, int n_steps, int sb
         if (item >= n_items) break;
         const int idx = item * G + g;
         const int s = idx < n_sched ? W.order[idx] : -1;
-        run_scene<LPS, FLAT, OPT, ARENA>(W, s, gl, pts, fr, th, th_old, tb, n_steps, step0, xch, sbytes, tmap, item);
+        run_scene<LPS, FLAT, OPT, ARENA, GP>(W, s, gl, pts, fr, th, th_old, tb, n_steps, step0, xch, sbytes, tmap, item);
     }
 }
+
+#ifndef NPX_STEP_DEVICE_CODE   // (npx_step_gp.cu takes the code above into kernels of its own)
 
 // Flat ground: up to 16 warps per block, 128 registers a thread.
 template <int LPS, bool OPT>
 __global__ void __launch_bounds__(512) step_kernel(const __grid_constant__ WorldDev W, int n_steps, int sbytes,
                                                    const __grid_constant__ CUtensorMap tmap) {
-    step_body<LPS, true, OPT, false>(W, n_steps, sbytes, &tmap);
+    step_body<LPS, true, OPT, false, false>(W, n_steps, sbytes, &tmap);
 }
 
 // Height maps keep more state (the map window and its origin): 168 registers a thread, up to 12
@@ -1794,7 +1889,7 @@ __global__ void __launch_bounds__(512) step_kernel(const __grid_constant__ World
 template <int LPS, bool OPT>
 __global__ void __maxnreg__(168) step_kernel_hm(const __grid_constant__ WorldDev W, int n_steps, int sbytes,
                                                 const __grid_constant__ CUtensorMap tmap) {
-    step_body<LPS, false, OPT, false>(W, n_steps, sbytes, &tmap);
+    step_body<LPS, false, OPT, false, false>(W, n_steps, sbytes, &tmap);
 }
 
 // Arenas (robots colliding with one another, 8 or 16 lanes per scene), with the friction options
@@ -1802,7 +1897,7 @@ __global__ void __maxnreg__(168) step_kernel_hm(const __grid_constant__ WorldDev
 template <int LPS, bool FLAT>
 __global__ void __maxnreg__(168) step_kernel_arena(const __grid_constant__ WorldDev W, int n_steps, int sbytes,
                                                    const __grid_constant__ CUtensorMap tmap) {
-    step_body<LPS, FLAT, true, true>(W, n_steps, sbytes, &tmap);
+    step_body<LPS, FLAT, true, true, false>(W, n_steps, sbytes, &tmap);
 }
 
 __global__ void advance_kernel(long long *step, int n) { *step += n; }
@@ -1826,7 +1921,7 @@ __global__ void __launch_bounds__(128) init_kernel(const __grid_constant__ World
     for (int j = lane; j < nl - 1; j += 32) th[j] = W.theta[j0 + j];
     __syncwarp();
     Shape sh;
-    shape_update<32>(W, s, p0, np, l0, nl, th, fr, pts, lane, sh);
+    shape_update<32, false>(W, s, p0, np, l0, nl, th, fr, pts, lane, sh);
     for (int i = lane; i < np; i += 32) W.kappa[p0 + i] = 0;
     if (lane == 0) {
         float q[4] = {quat[4 * s], quat[4 * s + 1], quat[4 * s + 2], quat[4 * s + 3]};
@@ -1867,7 +1962,7 @@ __global__ void __launch_bounds__(128) refresh_kernel(const __grid_constant__ Wo
     for (int j = lane; j < nl - 1; j += 32) th[j] = W.theta[j0 + j];
     __syncwarp();
     Shape sh;
-    shape_update<32>(W, s, p0, np, l0, nl, th, fr, pts, lane, sh);
+    shape_update<32, false>(W, s, p0, np, l0, nl, th, fr, pts, lane, sh);
     uint32_t sens = 0;   // contact sensors of the written contact flags
     for (int i = lane; i < np; i += 32) {
         if (!W.kappa[p0 + i]) continue;
@@ -1900,7 +1995,7 @@ __global__ void __launch_bounds__(32) points_kernel(const __grid_constant__ Worl
     for (int j = lane; j < nl - 1; j += 32) th[j] = W.theta[j0 + j];
     __syncwarp();
     Shape sh;
-    shape_update<32>(W, s, p0, np, l0, nl, th, fr, pts, lane, sh);
+    shape_update<32, false>(W, s, p0, np, l0, nl, th, fr, pts, lane, sh);
     const int S = W.S;
     const float c[3] = {W.st[ST_CX * S + s], W.st[ST_CY * S + s], W.st[ST_CZ * S + s]};
     const float q[4] = {W.st[ST_QW * S + s], W.st[ST_QX * S + s], W.st[ST_QY * S + s],
@@ -1995,7 +2090,7 @@ __global__ void __launch_bounds__(128) shape_cache_kernel(const __grid_constant_
     for (int j = lane; j < nl - 1; j += 32) th[j] = W.theta[j0 + j];
     __syncwarp();
     Shape sh;
-    shape_update<32>(W, s, p0, np, l0, nl, th, fr, pts, lane, sh);
+    shape_update<32, false>(W, s, p0, np, l0, nl, th, fr, pts, lane, sh);
     for (int l = lane; l < C.nl; l += 32) {
         float4 lq = make_float4(1.f, 0.f, 0.f, 0.f), lp = make_float4(0.f, 0.f, 0.f, 0.f);
         if (l < nl) {
@@ -2364,7 +2459,7 @@ __global__ void __launch_bounds__(128) kappa_refresh_kernel(const __grid_constan
         for (int j = lane; j < nl - 1; j += 32) th[j] = W.theta[j0 + j];
         __syncwarp();
         Shape sh;
-        shape_update<32>(W, s, p0, np, l0, nl, th, fr, pts, lane, sh);
+        shape_update<32, false>(W, s, p0, np, l0, nl, th, fr, pts, lane, sh);
         const RootState x = load_root(W, s);
         float R[9];
         quat_mat(x.q, R);
@@ -2536,13 +2631,14 @@ cudaError_t launch_permute_kappa(uint8_t *dst, const uint8_t *src, const int *pe
 // ------------------------------------------------------------------------ host-side launchers
 
 // per-scene shared memory of the step kernel: the slot, plus the height-map window on maps
-int step_slot_bytes(const WorldDev &W, int lps) {
-    return W.hm ? hm_win_offset(W.max_points, W.max_links, lps) + HM_AREA : slot_bytes(W.max_points, W.max_links, lps);
+static int step_slot_bytes(const WorldDev &W, int lps, int gp) {
+    return W.hm ? hm_win_offset(W.max_points, W.max_links, lps) + HM_AREA
+                : slot_bytes(W.max_points, W.max_links, lps) - (gp ? 16 * W.max_points : 0);
 }
 
-size_t step_smem_bytes(const WorldDev &W, int lps, int wpb) {
+static size_t step_smem_bytes(const WorldDev &W, int lps, int wpb, int gp) {
     // (height maps) 128 more bytes to align the slots' windows for TMA
-    return (size_t)wpb * (32 / lps) * (step_slot_bytes(W, lps) + (W.arena > 1 ? xch_bytes(W.max_chunks) : 0)) +
+    return (size_t)wpb * (32 / lps) * (step_slot_bytes(W, lps, gp) + (W.arena > 1 ? xch_bytes(W.max_chunks) : 0)) +
            (W.hm ? 128 : 0);
 }
 
@@ -2653,8 +2749,11 @@ static void *pick_step_opt(int lps, bool flat) {
 
 // the kernel for a world: flat or height maps, friction options compiled in only when used,
 // arenas (8 or 16 lanes per scene) in their own build
-static void *pick_step(const WorldDev &W, int lps) {
+static void *pick_step(const WorldDev &W, int lps, int gp) {
     const bool flat = W.hm == nullptr;
+    if (gp) {
+        return !flat || W.fric_mode || W.arena > 1 ? nullptr : step_gp_kernel(lps);
+    }
     if (W.arena > 1) {
         if (lps == 8) return flat ? (void *)step_kernel_arena<8, true> : (void *)step_kernel_arena<8, false>;
         if (lps == 16) return flat ? (void *)step_kernel_arena<16, true> : (void *)step_kernel_arena<16, false>;
@@ -2663,11 +2762,27 @@ static void *pick_step(const WorldDev &W, int lps) {
     return W.fric_mode ? pick_step_opt<true>(lps, flat) : pick_step_opt<false>(lps, flat);
 }
 
-int step_blocks_per_sm(const WorldDev &W, int lps, int wpb, cudaError_t *err) {
-    void *fn = pick_step(W, lps);
+bool step_fits_bare(const WorldDev &W, int lps, int wpb) {
+    void *fn = pick_step(W, lps, 0);
+    cudaFuncAttributes fa{};
+    int dev = 0, optin = 0;
+    if (!fn || cudaGetDevice(&dev) != cudaSuccess || cudaFuncGetAttributes(&fa, fn) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+        return false;
+    const int slot = ((16 * W.max_points + 56 * W.max_links + 15) & ~15) + 32 * ((W.max_points + lps - 1) / lps);
+    const size_t smem = (size_t)wpb * (32 / lps) *
+                            ((W.hm ? ((slot + 127) & ~127) + HM_AREA : slot) + (W.arena > 1 ? xch_bytes(W.max_chunks) : 0)) +
+                        (W.hm ? 128 : 0);
+    return smem <= (size_t)optin && wpb * 32 <= fa.maxThreadsPerBlock;
+}
+
+bool step_has_gp(const WorldDev &W, int lps) { return pick_step(W, lps, 1) != nullptr; }
+
+int step_blocks_per_sm(const WorldDev &W, int lps, int wpb, int gp, cudaError_t *err) {
+    void *fn = pick_step(W, lps, gp);
     *err = cudaSuccess;
     if (!fn) { *err = cudaErrorInvalidValue; return 0; }
-    const size_t smem = step_smem_bytes(W, lps, wpb);
+    const size_t smem = step_smem_bytes(W, lps, wpb, gp);
     // a shape over the per-block limit does not fit: report 0 blocks without a failing call (a
     // failed runtime call would leave an error behind for the next launch check to pick up)
     int dev = 0, optin = 0;
@@ -2690,13 +2805,13 @@ int step_blocks_per_sm(const WorldDev &W, int lps, int wpb, cudaError_t *err) {
 }
 
 cudaError_t launch_step(const WorldDev &W, const LaunchCfg &cfg, int n_steps, cudaStream_t st) {
-    void *fn = pick_step(W, cfg.lps);
-    if (!fn || cfg.wpb < 1 || cfg.wpb > 16 || cfg.blocks < 1) return cudaErrorInvalidValue;
+    void *fn = pick_step(W, cfg.lps, cfg.gp);
+    if (!fn || cfg.wpb < 1 || cfg.wpb > 16 || cfg.blocks < 1 || (cfg.gp && !W.pscr)) return cudaErrorInvalidValue;
     // the kernel's shared-memory limit was raised by step_blocks_per_sm for this shape
-    const size_t smem = step_smem_bytes(W, cfg.lps, cfg.wpb);
+    const size_t smem = step_smem_bytes(W, cfg.lps, cfg.wpb, cfg.gp);
     cudaError_t e = cudaMemsetAsync(W.queue, 0, sizeof(unsigned int), st);
     if (e != cudaSuccess) return e;
-    int sb = step_slot_bytes(W, cfg.lps);
+    int sb = step_slot_bytes(W, cfg.lps, cfg.gp);
     WorldDev w = W;
     CUtensorMap tm;
     if (W.hm_tma && W.hm_tmap_h) tm = *W.hm_tmap_h;
@@ -2763,3 +2878,4 @@ extern "C" int npx_window_wait_selftest(int *gave_up, int *completed, int *elaps
     *elapsed_us = h[2];
     return NPX_OK;
 }
+#endif

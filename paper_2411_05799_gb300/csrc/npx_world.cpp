@@ -111,6 +111,7 @@ struct npx_world {
     struct SizeClass {
         int start, count, max_points, max_links;   // slice of the schedule and its largest scene
         int qi;                                    // its work-queue counter
+        size_t poff = 0;                           // its part of the point scratch
         npx::LaunchCfg cfg;
     };
     std::vector<SizeClass> classes;
@@ -152,6 +153,11 @@ struct npx_world {
         unsigned long long cache_gen = ~0ull;
     } sg;
     unsigned long long state_gen = 0;   // counts the caller's state writes
+    // posed points of the scenes in flight, for chunked launches that keep them in global memory: one
+    // part per size class (they run concurrently)
+    float4 *pscr = nullptr;
+    size_t pscr_n = 0;
+    bool pscr_off = false;              // its allocation failed: points stay in the slots
     size_t alist_n = 0;                 // entries allocated for the arenas' pair lists
     CUtensorMap hm_tmap{};              // TMA map of the height maps (W.hm_tmap_h points here)
     // angular velocity and contact sensors are derived from the state: after a state write they
@@ -293,9 +299,15 @@ int check_flat(const Flat &f, int scene) {
     return NPX_OK;
 }
 
+// Joint updates every so many steps at least for points in global memory: an update writes and reads
+// every point.
+constexpr int kGpMinK = 20;
+
 // launch shape for the scenes of W's schedule (count of them): checks the lanes per scene against
-// the largest scene, and sizes the grid to what is resident and what is needed
-npx::LaunchCfg clamp_cfg_for(npx_world *w, const npx::WorldDev &W, int count, npx::LaunchCfg c, int *rc) {
+// the largest scene, and sizes the grid to what is resident and what is needed; chunked: for the
+// chunks of npx_world_step (the surrogate's launches are a few steps each)
+npx::LaunchCfg clamp_cfg_for(npx_world *w, const npx::WorldDev &W, int count, npx::LaunchCfg c, int *rc,
+                             bool chunked = true) {
     *rc = NPX_OK;
     if (W.arena > 1 && c.lps * W.arena > 32) {
         *rc = fail(NPX_ERANGE, "an arena of %d robots is one warp: at most %d lanes per scene", W.arena, 32 / W.arena);
@@ -307,18 +319,41 @@ npx::LaunchCfg clamp_cfg_for(npx_world *w, const npx::WorldDev &W, int count, np
         return c;
     }
     cudaError_t e;
-    int nb = npx::step_blocks_per_sm(W, c.lps, c.wpb, &e);
+    c.gp = 0;
+    if (!c.grid) c.blocks = 0;   // an automatic grid is sized anew
+    int nb = npx::step_blocks_per_sm(W, c.lps, c.wpb, 0, &e);
+    if (e != cudaSuccess) { *rc = fail(NPX_ECUDA, "occupancy query: %s", cudaGetErrorString(e)); return c; }
+    // a shape that fits but for the tree numbers in the slots runs with fewer warps per block (the
+    // results do not depend on them)
+    if (nb < 1 && npx::step_fits_bare(W, c.lps, c.wpb))
+        while (nb < 1 && c.wpb > 1 && e == cudaSuccess) nb = npx::step_blocks_per_sm(W, c.lps, --c.wpb, 0, &e);
     if (e != cudaSuccess) { *rc = fail(NPX_ECUDA, "occupancy query: %s", cudaGetErrorString(e)); return c; }
     if (nb < 1) { *rc = fail(NPX_ERANGE, "launch shape lps=%d wpb=%d does not fit on an SM", c.lps, c.wpb); return c; }
     const int per_block = c.wpb * (32 / c.lps);
     const int need = (count + per_block - 1) / per_block;
+    // Points in global memory where shared memory holds fewer blocks than the registers and not
+    // every scene of the world fits at once (an explicit grid is one of blocks with their points in
+    // the slots).
+    if (chunked && !c.grid && !w->pscr_off && npx::step_has_gp(W, c.lps) && W.K >= kGpMinK &&
+        (long long)w->S > (long long)nb * w->n_sm * per_block) {
+        const int nbg = npx::step_blocks_per_sm(W, c.lps, c.wpb, 1, &e);
+        if (e != cudaSuccess) { *rc = fail(NPX_ECUDA, "occupancy query: %s", cudaGetErrorString(e)); return c; }
+        if (nbg > nb) {
+            c.gp = 1;
+            nb = nbg;
+        }
+    }
     const int full = nb * w->n_sm;
     if (c.blocks <= 0 || c.blocks > full) c.blocks = full;
     c.blocks = std::max(1, std::min(c.blocks, need));
     return c;
 }
 
-npx::LaunchCfg clamp_cfg(npx_world *w, npx::LaunchCfg c, int *rc) { return clamp_cfg_for(w, w->W, w->S, c, rc); }
+npx::LaunchCfg clamp_cfg(npx_world *w, npx::LaunchCfg c, int *rc) {
+    return clamp_cfg_for(w, w->W, w->S, c, rc, false);
+}
+
+void clear_graphs(npx_world *w);
 
 // the world as one class's launch sees it: its slice of the schedule, its slot sizes and its own
 // work-queue counter (built from the current world, so that later changes -- actuators, state --
@@ -331,7 +366,51 @@ npx::WorldDev class_world(const npx_world *w, const npx_world::SizeClass &c) {
     W.max_points = c.max_points;
     W.max_links = c.max_links;
     W.queue = w->W.queue + c.qi;
+    W.pscr = w->pscr ? w->pscr + c.poff : nullptr;
     return W;
+}
+
+// points a class's launch shape keeps in global memory
+size_t scratch_points(const npx::LaunchCfg &c, int max_points) {
+    return c.gp ? (size_t)c.blocks * c.wpb * (32 / c.lps) * max_points : 0;
+}
+
+// Makes the point scratch hold n points; false when the memory is not there.  Launches that use the
+// old one have ended by then.
+bool scratch_grow(npx_world *w, size_t n) {
+    if (n <= w->pscr_n) return true;
+    cudaStreamSynchronize(w->stream);
+    clear_graphs(w);   // they hold its address
+    if (w->pscr) cudaFree(w->pscr);
+    w->pscr = nullptr;
+    w->pscr_n = 0;
+    void *p = nullptr;
+    if (cudaMalloc(&p, n * sizeof(float4)) != cudaSuccess) {
+        cudaGetLastError();
+        w->pscr_off = true;
+        return false;
+    }
+    w->pscr = static_cast<float4 *>(p);
+    w->pscr_n = n;
+    return true;
+}
+
+// Lays the point scratch out for the classes' launch shapes; without the memory for it they go back
+// to points in the slots.
+int scratch_fit(npx_world *w) {
+    size_t n = 0;
+    for (auto &c : w->classes) {
+        c.poff = n;
+        n += scratch_points(c.cfg, c.max_points);
+    }
+    if (scratch_grow(w, n)) return NPX_OK;
+    int rc = NPX_OK;
+    for (auto &c : w->classes) {
+        c.poff = 0;
+        c.cfg = clamp_cfg_for(w, class_world(w, c), c.count, {c.cfg.lps, c.cfg.wpb, 0}, &rc);
+        if (rc) return rc;
+    }
+    return NPX_OK;
 }
 
 // default shape for scenes of up to max_points points: the narrowest group that holds them,
@@ -410,16 +489,12 @@ int build_classes(npx_world *w, bool split) {
             c.max_points = std::max(c.max_points, pts(order[i]));
             c.max_links = std::max(c.max_links, lnk(order[i]));
         }
-        if (ranges.size() == 1) {
-            c.cfg = w->cfg;
-        } else {
-            int rc;
-            c.cfg = clamp_cfg_for(w, class_world(w, c), c.count, default_shape(c.max_points), &rc);
-            if (rc) return rc;
-        }
+        int rc;
+        c.cfg = clamp_cfg_for(w, class_world(w, c), c.count, ranges.size() == 1 ? w->cfg : default_shape(c.max_points), &rc);
+        if (rc) return rc;
         w->classes.push_back(c);
     }
-    return NPX_OK;
+    return scratch_fit(w);
 }
 
 void clear_graphs(npx_world *w) {
@@ -585,6 +660,7 @@ int npx_world_destroy(npx_world *w) {
         if (w->finalized) cudaStreamSynchronize(w->stream);
         clear_graphs(w);
         for (auto &b : w->bufs) cudaFree(b.p);
+        if (w->pscr) cudaFree(w->pscr);
     }
     if (w->sg.ev_w) cudaEventDestroy(w->sg.ev_w);
     if (w->sg.ev_n) cudaEventDestroy(w->sg.ev_n);
@@ -1087,6 +1163,7 @@ int npx_world_set_friction_model(npx_world *w, int flags) {
         }
         w->cfg = clamp_cfg(w, w->cfg, &rc);
         if (rc) return rc;
+        return scratch_fit(w);
     }
     return NPX_OK;
 }
@@ -1379,7 +1456,8 @@ int npx_world_info_get(npx_world *w, npx_world_info *o) {
     if (!o) return fail(NPX_EINVAL, "null info");
     o->n_scenes = w->S; o->n_links = w->L; o->n_joints = w->J; o->n_points = w->P;
     o->max_points = w->max_points; o->max_links = w->max_links;
-    o->lanes_per_scene = w->cfg.lps; o->warps_per_block = w->cfg.wpb; o->blocks = w->cfg.blocks;
+    const npx::LaunchCfg &shape = w->classes.size() == 1 ? w->classes[0].cfg : w->cfg;
+    o->lanes_per_scene = shape.lps; o->warps_per_block = shape.wpb; o->blocks = shape.blocks;
     o->chunk_steps = w->chunk; o->step = w->step; o->kernel_launches = w->launches;
     o->size_classes = (int)w->classes.size();
     o->hm_window_tma = w->W.hm_tma;
@@ -1399,6 +1477,7 @@ int npx_world_configure(npx_world *w, int lps, int wpb, int blocks, int chunk) {
         c.wpb = wpb;
     }
     c.blocks = blocks > 0 ? blocks : (lps || wpb ? 0 : c.blocks);
+    c.grid = blocks > 0 ? 1 : (lps || wpb ? 0 : c.grid);
     if (chunk < 0) return fail(NPX_EINVAL, "chunk must be >= 0");
     int rc;
     c = clamp_cfg(w, c, &rc);
@@ -1672,7 +1751,7 @@ int npx_world_autotune(npx_world *w, int n_steps, npx_world_info *out) {
     const int lps_list[4] = {4, 8, 16, 32};
     int rc_out = NPX_OK;
     for (auto &cls : w->classes) {
-        const npx::WorldDev CW = class_world(w, cls);
+        npx::WorldDev CW = class_world(w, cls);
         const npx::LaunchCfg saved = cls.cfg;
         npx::LaunchCfg best = saved;
         float best_ms = 1e30f;
@@ -1693,6 +1772,11 @@ int npx_world_autotune(npx_world *w, int n_steps, npx_world_info *out) {
                 int rc;
                 npx::LaunchCfg c = clamp_cfg_for(w, CW, cls.count, {lps, wpb, 0}, &rc);
                 if (rc) { g_err.clear(); continue; }
+                if (!scratch_grow(w, scratch_points(c, cls.max_points))) {
+                    c = clamp_cfg_for(w, CW, cls.count, {lps, wpb, 0}, &rc);
+                    if (rc) { g_err.clear(); continue; }
+                }
+                CW.pscr = w->pscr;   // trials run one at a time
                 float ms = 0.f;
                 bool ok = true;
                 for (int rep = 0; rep < 2 && ok; ++rep) {   // first run warms up
@@ -1731,10 +1815,10 @@ int npx_world_autotune(npx_world *w, int n_steps, npx_world_info *out) {
         npx::LaunchCfg c = clamp_cfg(w, {w->classes[0].cfg.lps, w->classes[0].cfg.wpb, 0}, &rc_cfg);
         if (rc_cfg) rc_out = rc_cfg;
         else w->cfg = c;
-        if (w->classes.size() == 1) w->classes[0].cfg = w->cfg;
         // the occupancy queries above may have lowered nothing, but the class shapes come last
         for (auto &cls : w->classes) clamp_cfg_for(w, class_world(w, cls), cls.count, cls.cfg, &rc_cfg);
     }
+    if (int rc = scratch_fit(w); rc && !rc_out) rc_out = rc;
     clear_graphs(w);
     if (int rc = npx_state_import(w, blob.data(), bytes)) return rc;
     if (rc_out) return rc_out;

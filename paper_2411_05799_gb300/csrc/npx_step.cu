@@ -222,10 +222,11 @@ __device__ __forceinline__ float asin_small(float x) {
 __host__ __device__ inline int tiles_offset(int max_points, int max_links) {
     return (16 * max_points + 58 * max_links + 15) & ~15;
 }
-// 16 spare bytes after the boxes: at shape updates their area holds the points' links, shifted by up
-// to 3 bytes
+// 16 spare bytes after the boxes (at shape updates their area holds the points' links, shifted by up
+// to 3 bytes), then the reference of the friction-set moments (from the boxes: ref_offset)
+__host__ __device__ inline int ref_offset(int max_points, int lps) { return 32 * ((max_points + lps - 1) / lps) + 16; }
 __host__ __device__ inline int slot_bytes(int max_points, int max_links, int lps) {
-    return tiles_offset(max_points, max_links) + 32 * ((max_points + lps - 1) / lps) + 16;
+    return tiles_offset(max_points, max_links) + ref_offset(max_points, lps) + 16;
 }
 // (height maps) the window and its mbarrier after the slot, 128-byte aligned for the TMA box
 __host__ __device__ inline int hm_win_offset(int max_points, int max_links, int lps) {
@@ -1337,6 +1338,8 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
     // and whether it has to be found again
     float ref[3] = {0.f, 0.f, 0.f};
     bool ref_any = false, ref_stale = true;
+    float4 *refc = reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(tb) +
+                                              ref_offset(W.max_points, LPS));   // (PIN: kept here)
     int ph = (int)(step0 % (long long)W.K);
     for (int t = 0; t < n_steps; ++t) {
         const long long n = step0 + t;
@@ -1467,11 +1470,31 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
         }
         // reference o of the friction-set moments: the rotated centre of the first tile holding a
         // point that was in contact last step (C is a subset of those; o depends on the state alone).
-        // On maps the tile's centre is kept until a scene of the warp changes its contacts or its
-        // shape: finding it is a chain of shuffles and shared-memory loads (rough terrain 8.81 us a
-        // step after, 9.09 before).
+        // The tile's centre is kept until a scene of the warp changes its contacts or its shape:
+        // finding it is a chain of shuffles and shared-memory loads (rough terrain 8.81 us a step
+        // after, 9.09 before).  On flat ground, where registers are short, it is kept in the slot
+        // (one hexapod, 100 steps: 141 -> 131 us; 4,096, 1,000 steps: 2.12 -> 2.09 ms).
         float o[3] = {0.f, 0.f, 0.f};
-        if constexpr (FLAT) {
+        if constexpr (PIN) {
+            if (__any_sync(FULL_MASK, ref_stale)) {
+                ref_stale = false;
+                int kf = kprev ? __ffsll((long long)kprev) - 1 : 64;
+#pragma unroll
+                for (int ofs = LPS / 2; ofs > 0; ofs >>= 1) kf = min(kf, __shfl_xor_sync(FULL_MASK, kf, ofs));
+                if (gl == 0) {
+                    float4 mid = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (kf < 64) {
+                        const float4 lo = tb[2 * kf], hi = tb[2 * kf + 1];
+                        mid = make_float4(0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z), 0.f);
+                    }
+                    *refc = mid;
+                }
+                __syncwarp();
+            }
+            const float4 mid = *refc;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) o[k] = pin3<PIN>(R[3 * k], mid.x, R[3 * k + 1], mid.y, R[3 * k + 2], mid.z);
+        } else if constexpr (FLAT) {
             int kf = kprev ? __ffsll((long long)kprev) - 1 : 64;
 #pragma unroll
             for (int ofs = LPS / 2; ofs > 0; ofs >>= 1) kf = min(kf, __shfl_xor_sync(FULL_MASK, kf, ofs));

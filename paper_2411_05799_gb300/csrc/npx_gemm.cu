@@ -170,6 +170,10 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ C
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    // all of the above before the kernel ahead has ended (this one's shared memory leaves no room
+    // for a second block, and so for a second TMEM allocation, on an SM)
+    early_next();
+    early_wait();
 
     if (warp == 0) {
         // ---- TMA producer
@@ -367,8 +371,7 @@ static cudaError_t launch(const CUtensorMap &ta, const CUtensorMap &tb, const CU
     if (e != cudaSuccess) return e;
     const int tiles = (M / BM) * (N / BN) * splits;
     const int grid = tiles < sm_count() ? tiles : sm_count();
-    gemm_tn_kernel<BN, STORE><<<grid, THREADS, smem, st>>>(ta, tb, tout, M, N, K / splits, splits, ep, err);
-    return cudaGetLastError();
+    return launch_early(gemm_tn_kernel<BN, STORE>, grid, THREADS, smem, st, ta, tb, tout, M, N, K / splits, splits, ep, err);
 }
 
 // The bounded barrier wait on its own: thread 0 waits on a barrier that nothing completes; with

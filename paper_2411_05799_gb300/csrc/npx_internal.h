@@ -217,3 +217,33 @@ __nv_bfloat16 *mlp_input(npx_mlp *net, int *ld);
 int mlp_forward_packed(npx_mlp *net, int M, int cols);
 const float *mlp_output(const npx_mlp *net, int *ld);
 }  // namespace npx
+
+#ifdef __CUDACC__
+#include <utility>
+
+namespace npx {
+// Programmatic dependent launch, for chains of short kernels on one stream: a kernel launched with
+// launch_early is set up and its blocks placed while the kernel before it still runs.  Every such
+// kernel calls early_wait before it touches memory that another kernel wrote or reads (it returns
+// when the kernel before, which itself waited for its own, has ended and its writes are visible),
+// and early_next where its successor may start.  A training step is 18 launches of 3 to 15 us: four
+// minibatches of 8,192 rows (271 -> 4 x 512 -> 247) 1,178 -> 1,025 us.
+__device__ __forceinline__ void early_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void early_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_early(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+}  // namespace npx
+#endif

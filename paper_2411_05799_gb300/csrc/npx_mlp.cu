@@ -33,6 +33,8 @@ int pad_to(int n, int m) { return (n + m - 1) / m * m; }
 __global__ void __launch_bounds__(256) pack_input_kernel(const float *__restrict__ x, int M, int n_in, int in_p,
                                                          bf16 *X, bf16 *XT) {
     __shared__ bf16 tile[32][33];
+    npx::early_next();
+    npx::early_wait();
     const int k0 = blockIdx.x * 32, m0 = blockIdx.y * 32, tx = threadIdx.x, ty = threadIdx.y;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -53,6 +55,8 @@ __global__ void __launch_bounds__(256) loss_grad_kernel(const float *__restrict_
                                                         float *loss) {
     __shared__ bf16 tile[32][33];
     __shared__ float red[8];
+    npx::early_next();
+    npx::early_wait();
     const int j0 = blockIdx.x * 32, m0 = blockIdx.y * 32, tx = threadIdx.x, ty = threadIdx.y;
     const float inv = 1.f / (float)M;
     float sq = 0.f;
@@ -102,6 +106,8 @@ __global__ void __launch_bounds__(256) grads_finish_kernel(const __grid_constant
     int k = 0;
     while (k + 1 < G.layers && (int)blockIdx.x >= G.l[k + 1].first) ++k;
     const GradLayer &g = G.l[k];
+    npx::early_next();
+    npx::early_wait();
     int blk = (int)blockIdx.x - g.first;
     if (blk >= g.rows) {   // four weights a thread
         const long long i = ((long long)(blk - g.rows) * 256 + threadIdx.x) * 4;
@@ -168,6 +174,8 @@ __global__ void __launch_bounds__(256) adam_kernel(const __grid_constant__ AdamG
     int k = 0;
     while (k + 1 < A.layers && (int)blockIdx.x >= A.l[k + 1].first) ++k;
     const AdamLayer &g = A.l[k];
+    npx::early_next();
+    npx::early_wait();
     const int blk = (int)blockIdx.x - g.first, tc = g.cols / 32, tiles = (g.rows / 32) * tc;
     if (blk >= tiles) {
         const int i = (blk - tiles) * 256 + threadIdx.x;
@@ -381,9 +389,8 @@ bool fused_net(const npx_mlp *n, npx::FusedNet *f) {
 
 int forward_impl(npx_mlp *n, const float *x, int M, bool train) {
     const int in_p = n->din[0];
-    pack_input_kernel<<<dim3(in_p / 32, M / 32), dim3(32, 8), 0, n->stream>>>(x, M, n->d.n_in, in_p, n->X0,
-                                                                             train ? n->X0T : nullptr);
-    CU(cudaGetLastError());
+    CU(npx::launch_early(pack_input_kernel, dim3(in_p / 32, M / 32), dim3(32, 8), 0, n->stream, x, M, n->d.n_in, in_p, n->X0,
+                         train ? n->X0T : nullptr));
     return forward_layers(n, M, train);
 }
 
@@ -558,9 +565,8 @@ int npx_mlp_backward(npx_mlp *n, const float *x, const float *t, int M, float *l
     RC(forward_impl(n, x, M, true));
     const int L = n->L, H = n->d.n_hidden, out_p = n->dout[L - 1];
     CU(cudaMemsetAsync(loss, 0, sizeof(float), n->stream));
-    loss_grad_kernel<<<dim3(out_p / 32, M / 32), dim3(32, 8), 0, n->stream>>>(n->Y, t, M, n->d.n_out, out_p, n->dY,
-                                                                              n->dYT, loss);
-    CU(cudaGetLastError());
+    CU(npx::launch_early(loss_grad_kernel, dim3(out_p / 32, M / 32), dim3(32, 8), 0, n->stream, n->Y, t, M, n->d.n_out, out_p,
+                         n->dY, n->dYT, loss));
     const bf16 *G = n->dY, *GT = n->dYT;     // gradient of the current layer's output
     GradGroup group;
     group.layers = 0;
@@ -579,8 +585,7 @@ int npx_mlp_backward(npx_mlp *n, const float *x, const float *t, int M, float *l
         g = GradLayer{splits > 1 ? n->part[l] : nullptr, n->dW[l], GT, n->db[l], splits, No, blocks, (long long)No * Ni};
         blocks += No + (splits > 1 ? (int)blocks_for(g.n / 4) : 0);
         if (group.layers == GROUP || l == 0) {
-            grads_finish_kernel<<<blocks, 256, 0, n->stream>>>(group, M);
-            CU(cudaGetLastError());
+            CU(npx::launch_early(grads_finish_kernel, blocks, 256, 0, n->stream, group, M));
             group.layers = 0;
             blocks = 0;
         }
@@ -631,12 +636,11 @@ int npx_mlp_adam_step(npx_mlp *n) {
                                     n->Wb[l], n->WbT[l], rows, cols, blocks};
         blocks += (rows / 32) * (cols / 32) + (int)blocks_for(rows);
         if (A.layers == GROUP || l == n->L - 1) {
-            adam_kernel<<<blocks, 256, 0, n->stream>>>(A);
+            CU(npx::launch_early(adam_kernel, blocks, 256, 0, n->stream, A));
             A.layers = 0;
             blocks = 0;
         }
     }
-    CU(cudaGetLastError());
     return NPX_OK;
 }
 

@@ -117,11 +117,38 @@ __device__ __forceinline__ void epilogue16(const npx_gemm_epilogue &ep, float (&
 
 // STORE = 2: the FP32 row-major output (outf) leaves through per-warp shared-memory boxes and TMA
 // stores (tout); STORE = 0: every output is stored directly.
-template <int BN, int STORE>
+// G products in one launch: their tiles (and split-K ranges) form one list, walked by the persistent
+// blocks, so that a product's epilogues run under the next one's copies and MMAs.
+template <int G>
+struct Products {
+    CUtensorMap a[G], b[G], out[G];
+    int tiles_n[G], k_per_split[G], splits[G], first[G];   // first: the product's place in the list
+    int n, total;
+};
+
+struct Tile {
+    int p, m0, n0, split, kbeg, nk;
+};
+
+template <int BN, int G>
+__device__ __forceinline__ Tile tile_at(const Products<G> &P, int t) {
+    Tile r;
+    r.p = 0;
+    if (G > 1)
+        while (r.p + 1 < P.n && t >= P.first[r.p + 1]) ++r.p;
+    t -= P.first[r.p];
+    const int splits = P.splits[r.p], tiles_n = P.tiles_n[r.p], rest = t / splits;
+    r.split = t % splits;
+    r.n0 = (rest % tiles_n) * BN;
+    r.m0 = (rest / tiles_n) * BM;
+    r.kbeg = r.split * P.k_per_split[r.p];
+    r.nk = P.k_per_split[r.p] / BK;
+    return r;
+}
+
+template <int BN, int STORE, int G>
 __global__ void __launch_bounds__(THREADS, 1)
-gemm_tn_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
-               const __grid_constant__ CUtensorMap tout, int M, int N, int k_per_split, int splits,
-               npx_gemm_epilogue ep, int *err) {
+gemm_tn_kernel(const __grid_constant__ Products<G> P, npx_gemm_epilogue ep, int *err) {
     constexpr int store_mode = STORE;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -142,8 +169,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ C
     uint8_t *stage_base = sB + STAGES * B_BYTES + 1024;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tiles_m = M / BM, tiles_n = N / BN, total = tiles_m * tiles_n * splits;
-    const int nk = k_per_split / BK;
+    const int total = P.total;
 
     if (warp == 1) {   // whole warp: allocate two accumulators of BN columns
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
@@ -181,18 +207,16 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ C
             int g = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-                const int split = t % splits, rest = t / splits;
-                const int n0 = (rest % tiles_n) * BN, m0 = (rest / tiles_n) * BM;
-                const int kbeg = split * k_per_split;
-                for (int kb = 0; kb < nk; ++kb, ++g) {
+                const Tile T = tile_at<BN>(P, t);
+                for (int kb = 0; kb < T.nk; ++kb, ++g) {
                     const int s = g % STAGES;
                     if (g >= STAGES && !mbar_wait(&empty[s], (uint32_t)(((g / STAGES) - 1) & 1), abort)) {
                         ok = false;
                         break;
                     }
                     mbar_expect_tx(&full[s], A_BYTES + B_BYTES);
-                    tma_load_2d(sA + s * A_BYTES, &ta, kbeg + kb * BK, m0, &full[s]);
-                    tma_load_2d(sB + s * B_BYTES, &tb, kbeg + kb * BK, n0, &full[s]);
+                    tma_load_2d(sA + s * A_BYTES, &P.a[T.p], T.kbeg + kb * BK, T.m0, &full[s]);
+                    tma_load_2d(sB + s * B_BYTES, &P.b[T.p], T.kbeg + kb * BK, T.n0, &full[s]);
                     *issued = g + 1;
                 }
             }
@@ -215,6 +239,7 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ C
                 }
                 tc_fence_after();
                 const uint32_t d = tmem + (uint32_t)(b * BN);
+                const int nk = tile_at<BN>(P, t).nk;
                 for (int kb = 0; kb < nk; ++kb, ++g) {
                     const int s = g % STAGES;
                     if (!mbar_wait(&full[s], (uint32_t)((g / STAGES) & 1), abort)) {
@@ -249,8 +274,8 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ C
         int tl = 0;
         for (int t = blockIdx.x; t < total; t += gridDim.x, ++tl) {
             const int b = tl & 1;
-            const int split = t % splits, rest = t / splits;
-            const int n0 = (rest % tiles_n) * BN, m0 = (rest / tiles_n) * BM;
+            const Tile T = tile_at<BN>(P, t);
+            const int n0 = T.n0, m0 = T.m0, split = T.split;
             if (!mbar_wait(&tfull[b], (uint32_t)((tl >> 1) & 1), abort)) {
                 if (lane == 0) {
                     *abort = 1;
@@ -286,8 +311,8 @@ gemm_tn_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ C
                     fence_async_shared();
                     __syncwarp();
                     if (lane == 0) {
-                        if (f32) tma_store_3d(&tout, n0 + c0, m0 + q * 32, split, box);
-                        else tma_store_2d(&tout, n0 + c0, m0 + q * 32, box);
+                        if (f32) tma_store_3d(&P.out[T.p], n0 + c0, m0 + q * 32, split, box);
+                        else tma_store_2d(&P.out[T.p], n0 + c0, m0 + q * 32, box);
                         bulk_commit();
                     }
                     ++nstore;
@@ -363,15 +388,50 @@ static int sm_count() {
     return n;
 }
 
-template <int BN, int STORE>
-static cudaError_t launch(const CUtensorMap &ta, const CUtensorMap &tb, const CUtensorMap &tout, int M, int N, int K,
-                          int splits, const npx_gemm_epilogue &ep, int *err, cudaStream_t st) {
+template <int BN, int STORE, int G>
+static cudaError_t launch(const Products<G> &P, const npx_gemm_epilogue &ep, int *err, cudaStream_t st) {
     const size_t smem = smem_bytes<BN, STORE>();
-    cudaError_t e = cudaFuncSetAttribute(gemm_tn_kernel<BN, STORE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(gemm_tn_kernel<BN, STORE, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int tiles = (M / BM) * (N / BN) * splits;
-    const int grid = tiles < sm_count() ? tiles : sm_count();
-    return launch_early(gemm_tn_kernel<BN, STORE>, grid, THREADS, smem, st, ta, tb, tout, M, N, K / splits, splits, ep, err);
+    const int grid = P.total < sm_count() ? P.total : sm_count();
+    return launch_early(gemm_tn_kernel<BN, STORE, G>, grid, THREADS, smem, st, P, ep, err);
+}
+
+// the product's place after those in P
+template <int G>
+static void append(Products<G> &P, int M, int N, int K, int splits, int BN) {
+    const int i = P.n++;
+    P.tiles_n[i] = N / BN;
+    P.k_per_split[i] = K / splits;
+    P.splits[i] = splits;
+    P.first[i] = P.total;
+    P.total += (M / BM) * (N / BN) * splits;
+}
+
+// products of one launch, and those of them with tiles BN wide
+constexpr int MAX_G = 8;
+
+template <int BN>
+static int run_group(const GemmF32 *p, int n, int *err, cudaStream_t st) {
+    Products<MAX_G> P;
+    P.n = P.total = 0;
+    npx_gemm_epilogue ep{};
+    ep.mode = NPX_EPI_F32;
+    for (int i = 0; i < n; ++i) {
+        if ((p[i].N % 256 == 0 ? 256 : 128) == BN) {
+            if (!make_map(&P.a[P.n], p[i].A, p[i].M, p[i].K, BM) || !make_map(&P.b[P.n], p[i].B, p[i].N, p[i].K, BN) ||
+                !make_out_map(&P.out[P.n], p[i].out, true, p[i].M, p[i].N, p[i].N, p[i].splits, (long long)p[i].M * p[i].N))
+                return set_last_error(NPX_ECUDA, "grouped product: tensor-map encoding failed");
+            append(P, p[i].M, p[i].N, p[i].K, p[i].splits, BN);
+            ep.outf = p[i].out;   // (stored through the maps)
+        }
+        if (P.n == MAX_G || (i == n - 1 && P.n)) {
+            cudaError_t e = launch<BN, 2>(P, ep, err, st);
+            if (e != cudaSuccess) return set_last_error(NPX_ECUDA, cudaGetErrorString(e));
+            P.n = P.total = 0;
+        }
+    }
+    return NPX_OK;
 }
 
 // The bounded barrier wait on its own: thread 0 waits on a barrier that nothing completes; with
@@ -422,6 +482,11 @@ extern "C" int npx_gemm_wait_selftest(int use_abort, int *timed_out, int *elapse
     return NPX_OK;
 }
 
+int npx::gemm_group(const GemmF32 *p, int n, int *err, cudaStream_t st) {
+    if (int rc = gemm::run_group<256>(p, n, err, st)) return rc;
+    return gemm::run_group<128>(p, n, err, st);
+}
+
 extern "C" int npx_gemm_bf16(const void *A, const void *B, int M, int N, int K, int splits,
                              const npx_gemm_epilogue *ep, int *err, void *stream) {
     using namespace npx::gemm;
@@ -447,8 +512,11 @@ extern "C" int npx_gemm_bf16(const void *A, const void *B, int M, int N, int K, 
         (ep->outT && (reinterpret_cast<uintptr_t>(ep->outT) & 1)))
         return npx::set_last_error(NPX_EINVAL, "npx_gemm_bf16: outputs, bias and zin need 16-byte aligned rows");
     if (splits > 1 && ep->mode != NPX_EPI_F32) return npx::set_last_error(NPX_EINVAL, "npx_gemm_bf16: split K needs the F32 epilogue");
-    CUtensorMap ta, tb, tout;
-    if (!make_map(&ta, A, M, K, BM) || !make_map(&tb, B, N, K, BN))
+    Products<1> P;
+    P.n = P.total = 0;
+    append(P, M, N, K, splits, BN);
+    CUtensorMap &tout = P.out[0];
+    if (!make_map(&P.a[0], A, M, K, BM) || !make_map(&P.b[0], B, N, K, BN))
         return npx::set_last_error(NPX_ECUDA, "npx_gemm_bf16: tensor-map encoding failed");
     // the row-major output leaves through per-warp staging boxes and TMA stores: FP32 (store
     // mode 2), or BF16 when it is the only row-major output (mode 1)
@@ -466,14 +534,11 @@ extern "C" int npx_gemm_bf16(const void *A, const void *B, int M, int N, int K, 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e;
     if (store_mode == 2)
-        e = BN == 256 ? launch<256, 2>(ta, tb, tout, M, N, K, splits, *ep, err, st)
-                      : launch<128, 2>(ta, tb, tout, M, N, K, splits, *ep, err, st);
+        e = BN == 256 ? launch<256, 2>(P, *ep, err, st) : launch<128, 2>(P, *ep, err, st);
     else if (store_mode == 1)
-        e = BN == 256 ? launch<256, 1>(ta, tb, tout, M, N, K, splits, *ep, err, st)
-                      : launch<128, 1>(ta, tb, tout, M, N, K, splits, *ep, err, st);
+        e = BN == 256 ? launch<256, 1>(P, *ep, err, st) : launch<128, 1>(P, *ep, err, st);
     else
-        e = BN == 256 ? launch<256, 0>(ta, tb, tout, M, N, K, splits, *ep, err, st)
-                      : launch<128, 0>(ta, tb, tout, M, N, K, splits, *ep, err, st);
+        e = BN == 256 ? launch<256, 0>(P, *ep, err, st) : launch<128, 0>(P, *ep, err, st);
     if (e != cudaSuccess) return npx::set_last_error(NPX_ECUDA, cudaGetErrorString(e));
     return NPX_OK;
 }

@@ -201,6 +201,14 @@ bool fused_fits(const FusedNet &net);
 // that is given; rows a multiple of 128
 cudaError_t launch_mlp_fused(const FusedNet &net, const float *x, int n_in, const __nv_bfloat16 *xb, float *y, int ldy,
                              int ncols, int rows, int *err, cudaStream_t st);
+// C = A B^T per product (A [M x K], B [N x K] BF16, 16-byte aligned; C [splits][M x N] FP32), with M
+// a multiple of 128, N of 128 and K of 64 splits: as few launches as the tile widths allow
+struct GemmF32 {
+    const void *A, *B;
+    float *out;
+    int M, N, K, splits;
+};
+int gemm_group(const GemmF32 *p, int n, int *err, cudaStream_t st);
 }  // namespace npx
 
 struct npx_mlp;

@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(256) loss_grad_kernel(const float *__restrict_
 // of the layer's transposed output gradient GT [rows x M] (read from the transpose so that every load
 // is a full line).  Bound by launches: layer by layer these were ten launches of 4 to 6 us each,
 // 49 us of a 357 us minibatch of 8,192 rows (271 -> 4 x 512 -> 247); with Adam's ten below as one, a
-// minibatch takes 294 us.
+// minibatch took 294 us.
 constexpr int GROUP = 16;
 struct GradLayer {
     const float *part;      // [splits][n], or NULL: the gradient is written already
@@ -568,27 +568,16 @@ int npx_mlp_backward(npx_mlp *n, const float *x, const float *t, int M, float *l
     CU(npx::launch_early(loss_grad_kernel, dim3(out_p / 32, M / 32), dim3(32, 8), 0, n->stream, n->Y, t, M, n->d.n_out, out_p,
                          n->dY, n->dYT, loss));
     const bf16 *G = n->dY, *GT = n->dYT;     // gradient of the current layer's output
-    GradGroup group;
-    group.layers = 0;
-    int blocks = 0;
+    std::vector<npx::GemmF32> wgrads;
+    std::vector<GradLayer> finish;
     for (int l = L - 1; l >= 0; --l) {
         const int No = n->dout[l], Ni = n->din[l];
         // dW = G^T X_prev: A = G^T [No x M], B = X_prev^T [Ni x M]
         const bf16 *XprevT = l > 0 ? n->XT[l - 1] : n->X0T;
         const int splits = pick_splits(No, Ni, M);
-        npx_gemm_epilogue e = epi(NPX_EPI_F32);
-        e.outf = splits > 1 ? n->part[l] : n->dW[l];
-        e.ldf = Ni;
-        e.split_stride = (long long)No * Ni;
-        RC(gemm(n, GT, XprevT, No, Ni, M, splits, e));
-        GradLayer &g = group.l[group.layers++];
-        g = GradLayer{splits > 1 ? n->part[l] : nullptr, n->dW[l], GT, n->db[l], splits, No, blocks, (long long)No * Ni};
-        blocks += No + (splits > 1 ? (int)blocks_for(g.n / 4) : 0);
-        if (group.layers == GROUP || l == 0) {
-            CU(npx::launch_early(grads_finish_kernel, blocks, 256, 0, n->stream, group, M));
-            group.layers = 0;
-            blocks = 0;
-        }
+        float *out = splits > 1 ? n->part[l] : n->dW[l];
+        wgrads.push_back(npx::GemmF32{GT, XprevT, out, No, Ni, M, splits});
+        finish.push_back(GradLayer{splits > 1 ? out : nullptr, n->dW[l], GT, n->db[l], splits, No, 0, (long long)No * Ni});
         if (l > 0) {
             // dZ_prev = (G W) * gelu'(Z_prev): A = G [M x No], B = W^T [Ni x No]
             npx_gemm_epilogue e2 = epi(NPX_EPI_DGELU);
@@ -602,6 +591,21 @@ int npx_mlp_backward(npx_mlp *n, const float *x, const float *t, int M, float *l
             G = n->dZ[l - 1];
             GT = n->dZT[l - 1];
         }
+    }
+    // The weight gradients together, after the chain that the others hang on.  One alone is a tile of
+    // a few K blocks for each SM, whose epilogue nothing hides: four minibatches of 8,192 rows
+    // (271 -> 4 x 512 -> 247) 1,025 -> 1,002 us.
+    RC(npx::gemm_group(wgrads.data(), L, n->err, n->stream));
+    for (int l = 0; l < L; l += GROUP) {
+        GradGroup group;
+        group.layers = std::min(GROUP, L - l);
+        int blocks = 0;
+        for (int k = 0; k < group.layers; ++k) {
+            GradLayer &g = group.l[k] = finish[l + k];
+            g.first = blocks;
+            blocks += g.rows + (g.part ? (int)blocks_for(g.n / 4) : 0);
+        }
+        CU(npx::launch_early(grads_finish_kernel, blocks, 256, 0, n->stream, group, M));
     }
     return NPX_OK;
 }

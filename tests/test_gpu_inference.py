@@ -154,3 +154,45 @@ def test_training_step(M, n_in, hidden, layers, n_out):
         n.backward(x.data_ptr(), t.data_ptr(), M, loss.data_ptr())
     for a, b in zip(sum(net.get_grads(), []), sum(other.get_grads(), [])):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("M,n_in,hidden,layers,n_out", [(128, 3, 128, 1, 2), (1152, 271, 256, 2, 129),
+                                                        (2048, 200, 256, 10, 300), (192 * 128, 40, 128, 2, 30)])
+def test_weight_gradients_together(M, n_in, hidden, layers, n_out):
+    """The layers' weight gradients come from as few launches as their widths allow (eight products
+    at most in one, 256 columns a tile apart from 128): each against the FP64 product of the BF16
+    arrays, taken by torch through the network's own formulas.  A BF16 array may differ from the
+    network's where an FP32 sum rounds the other way (half an ulp, 2^-9 of an element), and each of
+    the two arrays of a product passes through at most 2 (layers + 1) roundings: 2 (layers + 1) 2^-8
+    of the gradient's norm covers both."""
+    rng = np.random.default_rng(M + layers)
+    sizes = [n_in] + [hidden] * layers + [n_out]
+    Ws = [rng.normal(0, np.sqrt(2 / i), (o, i)).astype(np.float32) for i, o in zip(sizes[:-1], sizes[1:])]
+    bs = [rng.normal(0, 0.1, o).astype(np.float32) for o in sizes[1:]]
+    net = npx.MLP(n_in, n_out, n_hidden=hidden, n_hidden_layers=layers, max_batch=M,
+                  stream=torch.cuda.current_stream().cuda_stream)
+    net.set_params(Ws, bs)
+    x = torch.from_numpy(rng.normal(0, 1, (M, n_in)).astype(np.float32)).cuda()
+    t = torch.from_numpy(rng.normal(0, 1, (M, n_out)).astype(np.float32)).cuda()
+    loss = torch.zeros(1, device="cuda")
+    for _ in range(2):   # (the second pass right behind the first: nothing of it may be read early)
+        net.backward(x.data_ptr(), t.data_ptr(), M, loss.data_ptr())
+    torch.cuda.synchronize()
+    gWs, gbs = net.get_grads()
+    r = lambda a: a.to(torch.bfloat16).double()
+    W = [r(torch.from_numpy(w).cuda()) for w in Ws]
+    b = [torch.from_numpy(v).cuda().double() for v in bs]
+    X, Z = [r(x)], []
+    for l in range(layers):
+        z = X[-1] @ W[l].T + b[l]
+        Z.append(r(z))
+        X.append(r(torch.nn.functional.gelu(z, approximate="tanh")))
+    d = r(2.0 * (X[-1] @ W[-1].T + b[-1] - t.double()) / M)
+    for l in range(layers, -1, -1):
+        ref = d.T @ X[l]
+        err = (torch.from_numpy(gWs[l]).cuda().double() - ref).norm() / ref.norm()
+        assert float(err) <= 2 * (layers + 1) * 2.0 ** -8, (l, float(err))
+        if l:
+            z = Z[l - 1].clone().requires_grad_(True)
+            dg, = torch.autograd.grad(torch.nn.functional.gelu(z, approximate="tanh").sum(), z)
+            d = r((d @ W[l]) * dg)

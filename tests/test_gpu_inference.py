@@ -196,3 +196,32 @@ def test_weight_gradients_together(M, n_in, hidden, layers, n_out):
             z = Z[l - 1].clone().requires_grad_(True)
             dg, = torch.autograd.grad(torch.nn.functional.gelu(z, approximate="tanh").sum(), z)
             d = r((d @ W[l]) * dg)
+
+
+@pytest.mark.parametrize("mode", [npx.EPI_BIAS, npx.EPI_BIAS_GELU, npx.EPI_DGELU])
+@pytest.mark.parametrize("ldt, off", [(640, 0), (640, 1), (641, 0), (641, 1), (642, 2)])
+def test_transposed_output_on_any_address(mode, ldt, off):
+    """C^T goes out two rows to a store where its columns start on 4 bytes, one row otherwise: the same
+    values either way, nothing written beside them, and the transpose of the row-major output."""
+    M, N, K = 640, 384, 128
+    g = torch.Generator(device="cpu").manual_seed(ldt + off)
+    A = torch.randn(M, K, generator=g).to(torch.bfloat16).cuda()
+    B = torch.randn(N, K, generator=g).to(torch.bfloat16).cuda()
+    b = torch.randn(N, generator=g).cuda()
+    z = torch.randn(M, N, generator=g).to(torch.bfloat16).cuda()
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = torch.zeros(M, N, dtype=torch.bfloat16, device="cuda")
+    zs = torch.zeros(M, N, dtype=torch.bfloat16, device="cuda")
+    flat = torch.full((N * ldt + off,), 7.0, dtype=torch.bfloat16, device="cuda")
+    ep = npx.GemmEpilogue(mode=mode, bias=b.data_ptr() if mode != npx.EPI_DGELU else None, out=out.data_ptr(), ldo=N,
+                          outT=flat.data_ptr() + 2 * off, ldt=ldt,
+                          zsave=zs.data_ptr() if mode == npx.EPI_BIAS_GELU else None, ldz=N, zin=z.data_ptr(), ldzi=N)
+    npx.gemm_bf16(A.data_ptr(), B.data_ptr(), M, N, K, ep, err.data_ptr())
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    T = flat[off:].reshape(N, ldt)
+    assert torch.equal(T[:, :M], out.T)
+    assert (flat[:off] == 7.0).all() and (T[:, M:] == 7.0).all()
+    if mode == npx.EPI_BIAS_GELU:   # the pre-activations: FP32 sums of K products, rounded to BF16
+        ref = A.double() @ B.double().T + b.double()
+        assert ((zs.double() - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-4).all()

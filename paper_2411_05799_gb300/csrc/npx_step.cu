@@ -1473,7 +1473,7 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
         // The tile's centre is kept until a scene of the warp changes its contacts or its shape:
         // finding it is a chain of shuffles and shared-memory loads (rough terrain 8.81 us a step
         // after, 9.09 before).  On flat ground, where registers are short, it is kept in the slot
-        // (one hexapod, 100 steps: 141 -> 131 us; 4,096, 1,000 steps: 2.12 -> 2.09 ms).
+        // (one hexapod, 80 steps: 141 -> 131 us; 4,096, 1,000 steps: 2.12 -> 2.09 ms).
         float o[3] = {0.f, 0.f, 0.f};
         if constexpr (PIN) {
             if (__any_sync(FULL_MASK, ref_stale)) {

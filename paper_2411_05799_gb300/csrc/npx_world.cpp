@@ -333,12 +333,13 @@ npx::LaunchCfg clamp_cfg_for(npx_world *w, const npx::WorldDev &W, int count, np
     const int need = (count + per_block - 1) / per_block;
     // Points in global memory where shared memory holds fewer blocks than the registers and not
     // every scene of the world fits at once (an explicit grid is one of blocks with their points in
-    // the slots).
-    if (chunked && !c.grid && !w->pscr_off && npx::step_has_gp(W, c.lps) && W.K >= kGpMinK &&
+    // the slots): where that is half as many blocks again at least (352 points a scene: 2.3 times the
+    // blocks, 1.4 times the rate; 44 points, an eighth more blocks: 2.02 against 2.03e9 steps/s).
+    if (chunked && !c.grid && !c.slots && !w->pscr_off && npx::step_has_gp(W, c.lps) && W.K >= kGpMinK &&
         (long long)w->S > (long long)nb * w->n_sm * per_block) {
         const int nbg = npx::step_blocks_per_sm(W, c.lps, c.wpb, 1, &e);
         if (e != cudaSuccess) { *rc = fail(NPX_ECUDA, "occupancy query: %s", cudaGetErrorString(e)); return c; }
-        if (nbg > nb) {
+        if (2 * nbg >= 3 * nb) {
             c.gp = 1;
             nb = nbg;
         }
@@ -1749,6 +1750,11 @@ int npx_world_autotune(npx_world *w, int n_steps, npx_world_info *out) {
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));
     const int lps_list[4] = {4, 8, 16, 32};
+    // the largest scenes' fastest warps per block with points in the slots, per lanes per scene: the
+    // whole-world shape's (below), whose launches keep them there
+    int slot_wpb[33] = {0};
+    float slot_ms[33];
+    std::fill(slot_ms, slot_ms + 33, 1e30f);
     int rc_out = NPX_OK;
     for (auto &cls : w->classes) {
         npx::WorldDev CW = class_world(w, cls);
@@ -1768,12 +1774,20 @@ int npx_world_autotune(npx_world *w, int n_steps, npx_world_info *out) {
                 if (wb >= 1 && wb <= 16 && std::find(wpb_list.begin(), wpb_list.end(), wb) == wpb_list.end())
                     wpb_list.push_back(wb);
             }
-            for (int wpb : wpb_list) {
+            for (int k = 0; k < 2 * (int)wpb_list.size(); ++k) {   // as the rule has it, then in the slots
+                const int wpb = wpb_list[k / 2];
                 int rc;
                 npx::LaunchCfg c = clamp_cfg_for(w, CW, cls.count, {lps, wpb, 0}, &rc);
                 if (rc) { g_err.clear(); continue; }
                 if (!scratch_grow(w, scratch_points(c, cls.max_points))) {
                     c = clamp_cfg_for(w, CW, cls.count, {lps, wpb, 0}, &rc);
+                    if (rc) { g_err.clear(); continue; }
+                }
+                if (k & 1) {
+                    if (!c.gp) continue;   // the same shape again
+                    npx::LaunchCfg s{lps, wpb, 0};
+                    s.slots = 1;
+                    c = clamp_cfg_for(w, CW, cls.count, s, &rc);
                     if (rc) { g_err.clear(); continue; }
                 }
                 CW.pscr = w->pscr;   // trials run one at a time
@@ -1793,6 +1807,10 @@ int npx_world_autotune(npx_world *w, int n_steps, npx_world_info *out) {
                     cudaEventElapsedTime(&ms, e0, e1);
                 }
                 if (ok && ms < best_ms) { best_ms = ms; best = c; }
+                if (ok && !c.gp && &cls == &w->classes[0] && ms < slot_ms[lps]) {
+                    slot_ms[lps] = ms;
+                    slot_wpb[lps] = c.wpb;
+                }
                 if (!ok) {
                     rc_out = fail(NPX_ECUDA, "autotune trial lps=%d wpb=%d failed: %s", lps, wpb,
                                   cudaGetErrorString(cudaGetLastError()));
@@ -1812,7 +1830,8 @@ int npx_world_autotune(npx_world *w, int n_steps, npx_world_info *out) {
     // largest scenes
     if (!rc_out) {
         int rc_cfg;
-        npx::LaunchCfg c = clamp_cfg(w, {w->classes[0].cfg.lps, w->classes[0].cfg.wpb, 0}, &rc_cfg);
+        const npx::LaunchCfg &c0 = w->classes[0].cfg;
+        npx::LaunchCfg c = clamp_cfg(w, {c0.lps, slot_wpb[c0.lps] ? slot_wpb[c0.lps] : c0.wpb, 0}, &rc_cfg);
         if (rc_cfg) rc_out = rc_cfg;
         else w->cfg = c;
         // the occupancy queries above may have lowered nothing, but the class shapes come last

@@ -71,3 +71,19 @@ def test_shapes_at_the_edge_of_shared_memory():
         np.testing.assert_array_equal(r[k], ref[k], err_msg=k)
     with pytest.raises(NpxError):
         _after(b, (1,), lanes_per_scene=16, warps_per_block=fits + 1)
+
+
+def test_autotuned_shapes_agree():
+    """The autotuner times both homes of the points; what it settles on gives the bits of an explicit
+    grid with the same lanes."""
+    b = scenes.hexapod_batch(9001, seed_key=5)
+    w = World.from_batch(b)
+    lanes = w.autotune(20)["lanes_per_scene"]
+    ref = World.from_batch(b, configure=dict(lanes_per_scene=lanes, warps_per_block=1, blocks=152))
+    for x in (w, ref):
+        x.step(200)
+    r, q = w.read(), ref.read()
+    for k in KEYS:
+        np.testing.assert_array_equal(r[k], q[k], err_msg=k)
+    w.close()
+    ref.close()

@@ -421,7 +421,7 @@ def surrogate_leg(World, scenes, stream, device, n_transitions: int, stride: int
     flops = 2.0 * S * (n_in * H + (surrogate.N_LAYERS - 1) * H * H + H * n_out)
     peak = _measured_peaks().get("bf16_tflops")
     achieved = flops / (fwd_ms / 1e3) / 1e12
-    out["roofline"] = {"bound": "tensor", "kernel": "gemm_tn_kernel (network forward, 5 launches)",
+    out["roofline"] = {"bound": "tensor", "kernel": "mlp_fused_kernel (network forward)",
                        "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                        "frac": achieved / peak if peak else None, "traffic": None,
                        "flops_per_scene_step": flops / S,

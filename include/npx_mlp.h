@@ -59,6 +59,11 @@ int npx_gemm_bf16(const void *A, const void *B, int M, int N, int K, int splits,
  * the wait gave up, *elapsed_us (host) = how long it waited; the context stays usable. */
 int npx_gemm_wait_selftest(int use_abort, int *timed_out, int *elapsed_us, void *stream);
 
+/* The same wait by a whole warp, whose lanes go on or give up together: *split (host) = lanes told to
+ * go on when half of them wait on a barrier that has completed and half on one whose wait another
+ * warp aborts after 1 ms (0 expected), *complete = when all wait on the first (32).  Synchronous. */
+int npx_gemm_warp_wait_selftest(int *split, int *complete, void *stream);
+
 /* --- the surrogate network --------------------------------------------------------------
  * y = W_L gelu(... gelu(W_1 x + b_1) ...) + b_L with n_hidden_layers GELU layers of width
  * n_hidden (exact GELU, z Phi(z)), trained on the mean over the batch of the squared error summed

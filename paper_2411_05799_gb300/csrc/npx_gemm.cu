@@ -316,8 +316,7 @@ gemm_tn_kernel(const __grid_constant__ Products<G> P, npx_gemm_epilogue ep, int 
             if (ep.mode == NPX_EPI_DGELU) load_pair(zin, ep.ldzi, row, n0 + part * COLS, zn);
             if (ep.bias && lane < COLS / 32)
                 asm volatile("prefetch.global.L1 [%0];" ::"l"(ep.bias + n0 + part * COLS + 32 * lane));
-            // (the warp goes on or gives up as one: its lanes exchange values below)
-            if (!__all_sync(0xffffffffu, mbar_wait(&tfull[b], (uint32_t)((tl >> 1) & 1), abort))) {
+            if (!mbar_wait_warp(&tfull[b], (uint32_t)((tl >> 1) & 1), abort)) {
                 if (lane == 0) {
                     *abort = 1;
                     atomicExch(err, 3);
@@ -503,8 +502,57 @@ __global__ void __launch_bounds__(64) wait_selftest_kernel(int use_abort, int *o
     }
 }
 
+// A warp's wait whose lanes see different outcomes: the lower half waits on a barrier that has
+// completed, the upper half on one that nothing completes until warp 1 raises the abort flag.
+// out[0] = lanes told that they may go on, out[1] = the same when every lane's barrier has completed.
+__global__ void __launch_bounds__(64) warp_wait_selftest_kernel(int *out) {
+    __shared__ uint64_t bars[2];
+    __shared__ volatile int abort_flag;
+    if (threadIdx.x == 0) {
+        mbar_init(&bars[0], 1);
+        mbar_init(&bars[1], 1);
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        mbar_arrive(&bars[0]);
+    }
+    __syncthreads();
+    if (threadIdx.x == 32) {
+        const unsigned long long t0 = global_ns();
+        while (global_ns() - t0 < ABORT_NS) {
+        }
+        abort_flag = 1;
+    }
+    if (threadIdx.x < 32) {
+        const bool split = mbar_wait_warp(&bars[threadIdx.x >> 4], 0, &abort_flag);
+        const bool all = mbar_wait_warp(&bars[0], 0, &abort_flag);
+        const unsigned a = __ballot_sync(0xffffffffu, split), b = __ballot_sync(0xffffffffu, all);
+        if (threadIdx.x == 0) {
+            out[0] = __popc(a);
+            out[1] = __popc(b);
+        }
+    }
+}
+
 }  // namespace gemm
 }  // namespace npx
+
+extern "C" int npx_gemm_warp_wait_selftest(int *split, int *complete, void *stream) {
+    if (!split || !complete) return npx::set_last_error(NPX_EINVAL, "npx_gemm_warp_wait_selftest: null argument");
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    int *d = nullptr;
+    cudaError_t e = cudaMalloc(&d, 2 * sizeof(int));
+    if (e != cudaSuccess) return npx::set_last_error(NPX_ENOMEM, cudaGetErrorString(e));
+    int h[2] = {-1, -1};
+    npx::gemm::warp_wait_selftest_kernel<<<1, 64, 0, st>>>(d);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof h, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    cudaFree(d);
+    if (e != cudaSuccess) return npx::set_last_error(NPX_ECUDA, cudaGetErrorString(e));
+    *split = h[0];
+    *complete = h[1];
+    return NPX_OK;
+}
 
 extern "C" int npx_gemm_wait_selftest(int use_abort, int *timed_out, int *elapsed_us, void *stream) {
     if (!timed_out || !elapsed_us) return npx::set_last_error(NPX_EINVAL, "npx_gemm_wait_selftest: null argument");

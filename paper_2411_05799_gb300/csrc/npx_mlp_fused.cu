@@ -22,7 +22,8 @@
 // epilogue of each layer.  (Weights by cluster multicast, and pairs of CTAs sharing each MMA, which
 // halve or quarter the weights' traffic, measured no faster, 198 to 224 us, before those two: the
 // ring was not what it waited for.)
-// Waits are bounded as in npx_gemm.cu: a role that gives up sets the error flag and the others leave.
+// Waits are bounded as in npx_gemm.cu: a role that gives up sets the error flag and the others leave;
+// an epilogue warp goes on or gives up as one.
 #include <algorithm>
 #include <cstring>
 
@@ -195,7 +196,7 @@ mlp_fused_kernel(const __grid_constant__ FusedMaps maps, const __grid_constant__
         bool ok = true;
         for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++it) {
             // (the last tile's outputs were staged where these go)
-            if (it > 0 && !mbar_wait(freed, (uint32_t)((it - 1) & 1), abort)) {
+            if (it > 0 && !mbar_wait_warp(freed, (uint32_t)((it - 1) & 1), abort)) {
                 ok = false;
                 break;
             }
@@ -252,7 +253,7 @@ mlp_fused_kernel(const __grid_constant__ FusedMaps maps, const __grid_constant__
                 for (int n0 = 0; n0 < N; n0 += F_BN, ++step) {
                     const int b = step & 1, bn = min(F_BN, N - n0), nch = bn >> 6, c0 = part * (bn >> 2);
                     const bool last = n0 + F_BN >= N;
-                    if (!mbar_wait(&tfull[b], (uint32_t)((step >> 1) & 1), abort)) {
+                    if (!mbar_wait_warp(&tfull[b], (uint32_t)((step >> 1) & 1), abort)) {
                         ok = false;
                         break;
                     }
@@ -294,7 +295,7 @@ mlp_fused_kernel(const __grid_constant__ FusedMaps maps, const __grid_constant__
             // activations' memory can stage the rows for full-line stores
             const int N = net.n[L - 1], nb = (N + F_BN - 1) / F_BN;
             for (int j = 0; j < nb && ok; ++j)
-                if (!mbar_wait(&tfull[(step + j) & 1], (uint32_t)(((step + j) >> 1) & 1), abort)) ok = false;
+                if (!mbar_wait_warp(&tfull[(step + j) & 1], (uint32_t)(((step + j) >> 1) & 1), abort)) ok = false;
             if (!ok) break;
             tc_fence_after();
             // rows without padding between them are one block of memory: staged as they lie there, it
@@ -340,7 +341,8 @@ mlp_fused_kernel(const __grid_constant__ FusedMaps maps, const __grid_constant__
                 mbar_arrive(staged);
                 if (e == 0) {
                     if (!mbar_wait(staged, (uint32_t)(it & 1), abort)) {
-                        ok = false;
+                        *abort = 1;   // every warp gives up where it waits for freed
+                        atomicExch(err, 3);
                     } else {
                         if (bulk) {
                             asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(

@@ -54,6 +54,21 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity, const vo
     return true;
 }
 
+// The wait of a whole warp: true on every lane or on none.  A lane's own answer is not enough where
+// warp-wide instructions (tcgen05.ld, shuffles) follow: when another role raises the abort flag, or
+// the limit passes as the phase completes, some lanes see the phase and some the end of the wait.
+// (The votes cost the fused inference kernel about 1 of 137 us for 65,536 rows.)
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *b, uint32_t parity, const volatile int *abort = nullptr) {
+    bool ok = mbar_try_wait(b, parity);
+    if (__all_sync(0xffffffffu, ok)) return true;
+    const unsigned long long t0 = global_ns();
+    while (true) {
+        ok = ok || mbar_try_wait(b, parity);
+        if (__all_sync(0xffffffffu, ok)) return true;
+        if (__any_sync(0xffffffffu, (abort && *abort) || global_ns() - t0 > WAIT_NS)) return false;
+    }
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t *b) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
 }

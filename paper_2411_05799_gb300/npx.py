@@ -108,6 +108,15 @@ def gemm_wait_selftest(use_abort: bool, stream=None):
     return t.value, us.value
 
 
+def gemm_warp_wait_selftest(stream=None):
+    """npx_gemm_warp_wait_selftest: (lanes told to go on when half of a warp's barriers complete, when
+    all do)."""
+    load()
+    split, complete = C.c_int(), C.c_int()
+    _check(_lib.npx_gemm_warp_wait_selftest(C.byref(split), C.byref(complete), C.c_void_p(stream or 0)))
+    return split.value, complete.value
+
+
 def window_wait_selftest(stream=None):
     """The step kernel's bounded window-copy wait on its own: (lanes that gave up, lanes that saw
     their barrier complete, microseconds), two of its four 8-lane groups waiting on copies that are
@@ -156,6 +165,7 @@ _SIGS = {
     "npx_step_noalloc": [P, I, P],
     "npx_gemm_bf16": [P, P, I, I, I, I, P, P, P],
     "npx_gemm_wait_selftest": [I, P, P, P],
+    "npx_gemm_warp_wait_selftest": [P, P, P],
     "npx_window_wait_selftest": [P, P, P, P],
     "npx_world_set_friction_model": [P, I],
     "npx_world_set_arenas": [P, I, C.c_float],

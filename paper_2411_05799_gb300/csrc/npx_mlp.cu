@@ -30,17 +30,20 @@ int pad_to(int n, int m) { return (n + m - 1) / m * m; }
 // transpose are written in full lines: block (32, 8), grid (cols / 32, rows / 32).
 
 // X = bf16(x) zero-padded to in_p columns, and optionally X^T [in_p x M]
-__global__ void __launch_bounds__(256) pack_input_kernel(const float *__restrict__ x, int M, int n_in, int in_p,
+__global__ void __launch_bounds__(256) pack_input_kernel(const float *x, int M, int n_in, int in_p,
                                                          bf16 *X, bf16 *XT) {
     __shared__ bf16 tile[32][33];
     npx::early_next();
     npx::early_wait();
     const int k0 = blockIdx.x * 32, m0 = blockIdx.y * 32, tx = threadIdx.x, ty = threadIdx.y;
+    const int k = k0 + tx;
+    float f[4];   // (all loads first)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) f[i] = k < n_in ? x[(size_t)(m0 + ty + 8 * i) * n_in + k] : 0.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const int m = m0 + ty + 8 * i, k = k0 + tx;
-        const bf16 v = __float2bfloat16_rn(k < n_in ? x[(size_t)m * n_in + k] : 0.f);
-        X[(size_t)m * in_p + k] = v;
+        const bf16 v = __float2bfloat16_rn(f[i]);
+        X[(size_t)(m0 + ty + 8 * i) * in_p + k] = v;
         tile[ty + 8 * i][tx] = v;
     }
     if (!XT) return;   // block-uniform
@@ -50,9 +53,8 @@ __global__ void __launch_bounds__(256) pack_input_kernel(const float *__restrict
 }
 
 // dY = 2 (y - t) / M on real outputs, 0 on the padding, and dY^T; loss += sum (y - t)^2 / M
-__global__ void __launch_bounds__(256) loss_grad_kernel(const float *__restrict__ Y, const float *__restrict__ T,
-                                                        int M, int n_out, int out_p, bf16 *dY, bf16 *dYT,
-                                                        float *loss) {
+__global__ void __launch_bounds__(256) loss_grad_kernel(const float *Y, const float *T, int M, int n_out, int out_p,
+                                                        bf16 *dY, bf16 *dYT, float *loss) {
     __shared__ bf16 tile[32][33];
     __shared__ float red[8];
     npx::early_next();
@@ -60,13 +62,20 @@ __global__ void __launch_bounds__(256) loss_grad_kernel(const float *__restrict_
     const int j0 = blockIdx.x * 32, m0 = blockIdx.y * 32, tx = threadIdx.x, ty = threadIdx.y;
     const float inv = 1.f / (float)M;
     float sq = 0.f;
+    const int j = j0 + tx;
+    float y[4], t4[4];   // (all loads first)
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const int m = m0 + ty + 8 * i, j = j0 + tx;
-        const float d = j < n_out ? Y[(size_t)m * out_p + j] - T[(size_t)m * n_out + j] : 0.f;
+        const size_t m = m0 + ty + 8 * i;
+        y[i] = j < n_out ? Y[m * out_p + j] : 0.f;
+        t4[i] = j < n_out ? T[m * n_out + j] : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float d = y[i] - t4[i];
         sq += d * d * inv;
         const bf16 g = __float2bfloat16_rn(2.f * d * inv);
-        dY[(size_t)m * out_p + j] = g;
+        dY[(size_t)(m0 + ty + 8 * i) * out_p + j] = g;
         tile[ty + 8 * i][tx] = g;
     }
     __syncthreads();

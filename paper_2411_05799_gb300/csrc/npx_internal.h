@@ -112,6 +112,7 @@ struct LaunchCfg {
     int gp = 0;   // 1: the scenes' posed points in global memory (WorldDev::pscr), not in the slots
     int grid = 0; // 1: the caller asked for this grid size
     int slots = 0;  // 1: points stay in the slots (the autotuner timed that as the faster one)
+    int gp_steps = 0;   // (gp) launches of fewer steps keep the points in the slots
 };
 
 int step_blocks_per_sm(const WorldDev &W, int lps, int wpb, int gp, cudaError_t *err);

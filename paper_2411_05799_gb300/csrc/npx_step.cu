@@ -475,9 +475,7 @@ __device__ __noinline__ void shape_update(const WorldDev &W, int s, int p0, int 
     __syncwarp();
     const float gref[3] = {W.gref[3 * s], W.gref[3 * s + 1], W.gref[3 * s + 2]};
     float a[10] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-    for (int i = gl; i < np; i += LPS) {
-        const float4 q = GP ? W.p0m[p0 + i] : pts[i];
+    auto pose = [&](int i, const float4 &q) {
         float p[3];
         fk_point(fr, q, lk[i], p);
         const float dx = p[0] - gref[0], dy = p[1] - gref[1], dz = p[2] - gref[2], m = q.w;
@@ -486,6 +484,23 @@ __device__ __noinline__ void shape_update(const WorldDev &W, int s, int p0, int 
         a[1] += m * dx; a[2] += m * dy; a[3] += m * dz;
         a[4] += m * dx * dx; a[5] += m * dy * dy; a[6] += m * dz * dz;
         a[7] += m * dx * dy; a[8] += m * dx * dz; a[9] += m * dy * dz;
+    };
+    // GP: a load of one point must not pass the store of another, both in global memory, so the loads
+    // of several points go first by hand: one after the other they took 20 us or more of an entry or a
+    // joint update (11,000 hexapods, calls of one step: 114 us before, 77 after, 70 in the slots)
+    constexpr int AHEAD = 8;
+    if constexpr (GP) {
+        for (int i0 = gl; i0 < np; i0 += AHEAD * LPS) {
+            float4 q[AHEAD];
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) q[u] = W.p0m[p0 + min(i0 + u * LPS, np - 1)];
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u)
+                if (i0 + u * LPS < np) pose(i0 + u * LPS, q[u]);
+        }
+    } else {
+#pragma unroll 4
+        for (int i = gl; i < np; i += LPS) pose(i, pts[i]);
     }
     gsum<LPS, 10>(a);
     const float M = a[0], dx = a[1] / M, dy = a[2] / M, dz = a[3] / M;
@@ -502,10 +517,22 @@ __device__ __noinline__ void shape_update(const WorldDev &W, int s, int p0, int 
     sh.Ib.xz = -a[8] + M * dx * dz;
     sh.Ib.yz = -a[9] + M * dy * dz;
     sh.Ii = sym_inv(sh.Ib);
-    for (int i = gl; i < np; i += LPS) {
-        float4 r = pts[i];
-        r.x -= dx; r.y -= dy; r.z -= dz;
-        pts[i] = r;
+    if constexpr (GP) {
+        for (int i0 = gl; i0 < np; i0 += AHEAD * LPS) {
+            float4 r[AHEAD];
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u) r[u] = pts[min(i0 + u * LPS, np - 1)];
+#pragma unroll
+            for (int u = 0; u < AHEAD; ++u)
+                if (i0 + u * LPS < np)
+                    pts[i0 + u * LPS] = make_float4(r[u].x - dx, r[u].y - dy, r[u].z - dz, r[u].w);
+        }
+    } else {
+        for (int i = gl; i < np; i += LPS) {
+            float4 r = pts[i];
+            r.x -= dx; r.y -= dy; r.z -= dz;
+            pts[i] = r;
+        }
     }
     __syncwarp();
 }

@@ -113,6 +113,7 @@ struct npx_world {
         int qi;                                    // its work-queue counter
         size_t poff = 0;                           // its part of the point scratch
         npx::LaunchCfg cfg;
+        npx::LaunchCfg few;                        // launches of fewer than cfg.gp_steps steps
     };
     std::vector<SizeClass> classes;
     // classes run concurrently on the world's stream and up to kAuxStreams more (forked and joined
@@ -299,9 +300,14 @@ int check_flat(const Flat &f, int scene) {
     return NPX_OK;
 }
 
-// Joint updates every so many steps at least for points in global memory: an update writes and reads
-// every point.
-constexpr int kGpMinK = 20;
+// Points in global memory: an entry or a joint update writes and reads every point there, so joint
+// updates come every kGpMinK steps at least.  Where the last of the scenes in flight would be few (up
+// to 1.3 times what fits at once) those few wait for memory alone, and scenes of more than
+// kGpManyPoints points have little to gain; there updates come every kGpMinKTail steps at least and
+// launches are of kGpMinSteps steps or more.  Hexapods, 8 lanes, 9,728 at once, against the slots:
+// 10,500 of them, K = 20, 1,000 steps 0.86 times the rate, K = 40 0.97, K = 80 1.14; K = 80, calls of
+// 1, 8, 16 steps 0.79, 0.94, 1.09; 9,000 of them, K = 20 1.30, calls of 1, 8, 16 steps 1.07, 1.15, 1.25.
+constexpr int kGpMinK = 20, kGpMinKTail = 40, kGpMinSteps = 16, kGpManyPoints = 512;
 
 // launch shape for the scenes of W's schedule (count of them): checks the lanes per scene against
 // the largest scene, and sizes the grid to what is resident and what is needed; chunked: for the
@@ -319,7 +325,7 @@ npx::LaunchCfg clamp_cfg_for(npx_world *w, const npx::WorldDev &W, int count, np
         return c;
     }
     cudaError_t e;
-    c.gp = 0;
+    c.gp = c.gp_steps = 0;
     if (!c.grid) c.blocks = 0;   // an automatic grid is sized anew
     int nb = npx::step_blocks_per_sm(W, c.lps, c.wpb, 0, &e);
     if (e != cudaSuccess) { *rc = fail(NPX_ECUDA, "occupancy query: %s", cudaGetErrorString(e)); return c; }
@@ -339,8 +345,11 @@ npx::LaunchCfg clamp_cfg_for(npx_world *w, const npx::WorldDev &W, int count, np
         (long long)w->S > (long long)nb * w->n_sm * per_block) {
         const int nbg = npx::step_blocks_per_sm(W, c.lps, c.wpb, 1, &e);
         if (e != cudaSuccess) { *rc = fail(NPX_ECUDA, "occupancy query: %s", cudaGetErrorString(e)); return c; }
-        if (2 * nbg >= 3 * nb) {
+        const long long once = (long long)nbg * w->n_sm * per_block;
+        const bool tail = (w->S > once && 10ll * w->S < 13 * once) || W.max_points > kGpManyPoints;
+        if (2 * nbg >= 3 * nb && (!tail || W.K >= kGpMinKTail)) {
             c.gp = 1;
+            c.gp_steps = tail ? kGpMinSteps : 0;
             nb = nbg;
         }
     }
@@ -397,18 +406,23 @@ bool scratch_grow(npx_world *w, size_t n) {
 }
 
 // Lays the point scratch out for the classes' launch shapes; without the memory for it they go back
-// to points in the slots.
+// to points in the slots.  Sets the shapes of the launches of few steps.
 int scratch_fit(npx_world *w) {
     size_t n = 0;
     for (auto &c : w->classes) {
         c.poff = n;
         n += scratch_points(c.cfg, c.max_points);
     }
-    if (scratch_grow(w, n)) return NPX_OK;
+    const bool fits = scratch_grow(w, n);
     int rc = NPX_OK;
     for (auto &c : w->classes) {
-        c.poff = 0;
-        c.cfg = clamp_cfg_for(w, class_world(w, c), c.count, {c.cfg.lps, c.cfg.wpb, 0}, &rc);
+        npx::LaunchCfg slots{c.cfg.lps, c.cfg.wpb, 0};
+        slots.slots = 1;
+        if (!fits) {
+            c.poff = 0;
+            c.cfg = clamp_cfg_for(w, class_world(w, c), c.count, {c.cfg.lps, c.cfg.wpb, 0}, &rc);
+        }
+        c.few = c.cfg.gp_steps ? clamp_cfg_for(w, class_world(w, c), c.count, slots, &rc) : c.cfg;
         if (rc) return rc;
     }
     return NPX_OK;
@@ -525,7 +539,8 @@ int enqueue_steps(npx_world *w, int n) {
         for (int i = 0; i < nk; ++i) {
             const auto &c = w->classes[i];
             const int k = na > 0 ? i % (na + 1) : 0;
-            CUDA_TRY(npx::launch_step(class_world(w, c), c.cfg, nc, k == 0 ? w->stream : w->aux[k - 1]));
+            CUDA_TRY(npx::launch_step(class_world(w, c), nc < c.cfg.gp_steps ? c.few : c.cfg, nc,
+                                      k == 0 ? w->stream : w->aux[k - 1]));
         }
         for (int a = 0; a < na; ++a) {
             CUDA_TRY(cudaEventRecord(w->ev_join[a], w->aux[a]));

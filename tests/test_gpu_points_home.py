@@ -1,0 +1,80 @@
+"""Where a large world's posed points live: in global memory where that is the faster home, in shared
+memory elsewhere, with the same results."""
+import numpy as np
+import pytest
+
+from paper_2411_05799_gb300 import scenes
+from paper_2411_05799_gb300.npx import World
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+KEYS = ("cog", "quat", "vel", "omega", "angmom", "theta", "contacts", "status")
+
+
+def _pair(b, lanes, warps, stream=None):
+    """The world as the library lays it out, and with an explicit grid: points in shared memory."""
+    shape = dict(lanes_per_scene=lanes, warps_per_block=warps)
+    return [World.from_batch(b, stream=stream, configure=dict(shape, **kw)) for kw in ({}, {"blocks": 100000})]
+
+
+def _global(pair):
+    """Points in global memory: more blocks run at once than have room in shared memory."""
+    free, slots = (w.info()["blocks"] for w in pair)
+    return free > slots
+
+
+def _close(pair):
+    for w in pair:
+        w.close()
+
+
+@pytest.mark.parametrize("robots, K, home", [
+    (9000, 20, True), (9000, 19, False),              # all at once
+    (10500, 20, False), (10500, 39, False), (10500, 40, True),   # a last wave of few
+    (13000, 20, True)])                               # a last wave of many
+def test_joint_updates_decide_the_home(robots, K, home):
+    pair = _pair(scenes.legged_batch(robots, 6, seed_key=3, K=K), 8, 2)
+    assert _global(pair) == home
+    _close(pair)
+
+
+def test_calls_of_few_and_of_many_steps():
+    """Either side of the fewest steps that take the points to global memory, after one another, with
+    and without captured graphs: bit for bit the explicit grid's."""
+    b = scenes.legged_batch(10500, 6, seed_key=4, K=40)
+    pair = _pair(b, 8, 2)
+    assert _global(pair)
+    for graphs in (True, False):
+        for w in pair:
+            w.use_graphs(graphs)
+            for n in (16, 1, 15, 16, 17, 40, 3):
+                w.step(n)
+        r, q = (w.read() for w in pair)
+        for k in KEYS:
+            np.testing.assert_array_equal(r[k], q[k], err_msg=k)
+        np.testing.assert_array_equal(pair[0].contacts(), pair[1].contacts())
+    _close(pair)
+
+
+@pytest.mark.parametrize("robots", [9000, 11000, 16000])
+def test_single_steps_are_not_slower_for_it(robots):
+    """Calls of one step: within 1.25 times the time with the points in shared memory (the best of many
+    runs; on the way to this rule 11,000 robots took 1.6 times)."""
+    s = torch.cuda.Stream()
+    pair = _pair(scenes.legged_batch(robots, 6, seed_key=3, K=80), 8, 2, s.cuda_stream)
+    best = [1e9, 1e9]
+    for w in pair:
+        w.step(201)
+        w.sync()
+    for _ in range(30):
+        for i, w in enumerate(pair):
+            a, e = torch.cuda.Event(True), torch.cuda.Event(True)
+            a.record(s)
+            for _ in range(4):
+                w.step(1)
+            e.record(s)
+            e.synchronize()
+            best[i] = min(best[i], a.elapsed_time(e))
+    assert best[0] < 1.25 * best[1], best
+    _close(pair)

@@ -450,7 +450,7 @@ static void append(Products<G> &P, int M, int N, int K, int splits, int BN) {
 }
 
 // products of one launch, and those of them with tiles BN wide
-constexpr int MAX_G = 8;
+constexpr int MAX_G = GEMM_GROUP;
 
 template <int BN>
 static int run_group(const GemmF32 *p, int n, int *err, cudaStream_t st) {

@@ -210,6 +210,7 @@ struct GemmF32 {
     float *out;
     int M, N, K, splits;
 };
+constexpr int GEMM_GROUP = 8;   // products of one launch at most
 int gemm_group(const GemmF32 *p, int n, int *err, cudaStream_t st);
 }  // namespace npx
 

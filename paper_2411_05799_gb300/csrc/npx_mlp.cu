@@ -91,13 +91,13 @@ __global__ void __launch_bounds__(256) loss_grad_kernel(const float *Y, const fl
     }
 }
 
-// What is left of a backward pass for up to GROUP layers in one launch: the split-K partials of each
+// What is left of a backward pass for up to WGROUP layers in one launch: the split-K partials of each
 // weight gradient summed in split order, and each bias gradient, the sum over the M entries of a row
 // of the layer's transposed output gradient GT [rows x M] (read from the transpose so that every load
 // is a full line).  Bound by launches: layer by layer these were ten launches of 4 to 6 us each,
 // 49 us of a 357 us minibatch of 8,192 rows (271 -> 4 x 512 -> 247); with Adam's ten below as one, a
 // minibatch took 294 us.
-constexpr int GROUP = 16;
+constexpr int WGROUP = npx::GEMM_GROUP;   // layers whose weight gradients are formed together
 struct GradLayer {
     const float *part;      // [splits][n], or NULL: the gradient is written already
     float *dW;
@@ -107,7 +107,7 @@ struct GradLayer {
     long long n;
 };
 struct GradGroup {
-    GradLayer l[GROUP];
+    GradLayer l[WGROUP];
     int layers;
 };
 
@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(256) grads_finish_kernel(const __grid_constant
     }
 }
 
+constexpr int GROUP = 16;
 // Adam on FP32 master parameters of up to GROUP layers in one launch.  A block takes a 32 x 32 tile
 // of a weight matrix, so that the refreshed BF16 copy and, through shared memory, its transpose are
 // both written in full lines (element by element the transpose wrote two bytes to a sector), or 256
@@ -300,7 +301,10 @@ struct npx_mlp {
     std::vector<bf16 *> Wb, WbT;
     bf16 *X0 = nullptr, *X0T = nullptr, *dY = nullptr, *dYT = nullptr;
     std::vector<bf16 *> Z, X, XT, dZ, dZT;      // hidden layers
-    std::vector<float *> part;                  // split-K partials of each layer's weight gradient
+    // split-K partials of the layers' weight gradients: one buffer, which each WGROUP layers use anew
+    // (64 bytes a weight of a 512 x 512 layer: a buffer of every layer's own would be three quarters
+    // of a deep network's memory)
+    float *part = nullptr;
     float *Y = nullptr, *loss_tmp = nullptr;
     int *err = nullptr;
     int t = 0;
@@ -459,15 +463,21 @@ int npx_mlp_create(const npx_mlp_desc *d, npx_mlp **out) {
     bool ok = true;
     n->W.resize(n->L); n->b.resize(n->L); n->mW.resize(n->L); n->vW.resize(n->L); n->mb.resize(n->L);
     n->vb.resize(n->L); n->dW.resize(n->L); n->db.resize(n->L); n->Wb.resize(n->L); n->WbT.resize(n->L);
-    n->part.resize(n->L);
     for (int l = 0; l < n->L && ok; ++l) {
         const size_t nw = (size_t)n->dout[l] * n->din[l];
-        const int ms = pick_splits(n->dout[l], n->din[l], 0);
         ok = dalloc(n, &n->W[l], nw) && dalloc(n, &n->mW[l], nw) && dalloc(n, &n->vW[l], nw) &&
              dalloc(n, &n->dW[l], nw) && dalloc(n, &n->Wb[l], nw) && dalloc(n, &n->WbT[l], nw) &&
-             dalloc(n, &n->part[l], ms > 1 ? ms * nw : 0) && dalloc(n, &n->b[l], n->dout[l]) && dalloc(n, &n->mb[l], n->dout[l]) &&
+             dalloc(n, &n->b[l], n->dout[l]) && dalloc(n, &n->mb[l], n->dout[l]) &&
              dalloc(n, &n->vb[l], n->dout[l]) && dalloc(n, &n->db[l], n->dout[l]);
     }
+    size_t parts = 0, group = 0;   // (in the order of the backward pass, at the most splits of any batch)
+    for (int l = n->L - 1; l >= 0; --l) {
+        const int ms = pick_splits(n->dout[l], n->din[l], 0);
+        if ((n->L - 1 - l) % WGROUP == 0) group = 0;
+        group += ms > 1 ? (size_t)ms * n->dout[l] * n->din[l] : 0;
+        parts = std::max(parts, group);
+    }
+    ok = ok && dalloc(n, &n->part, parts);
     n->Z.resize(n->L - 1); n->X.resize(n->L - 1); n->XT.resize(n->L - 1); n->dZ.resize(n->L - 1); n->dZT.resize(n->L - 1);
     for (int l = 0; l < n->L - 1 && ok; ++l)
         ok = dalloc(n, &n->Z[l], (size_t)Mx * H) && dalloc(n, &n->X[l], (size_t)Mx * H) &&
@@ -579,12 +589,15 @@ int npx_mlp_backward(npx_mlp *n, const float *x, const float *t, int M, float *l
     const bf16 *G = n->dY, *GT = n->dYT;     // gradient of the current layer's output
     std::vector<npx::GemmF32> wgrads;
     std::vector<GradLayer> finish;
+    float *part = n->part;
     for (int l = L - 1; l >= 0; --l) {
         const int No = n->dout[l], Ni = n->din[l];
         // dW = G^T X_prev: A = G^T [No x M], B = X_prev^T [Ni x M]
         const bf16 *XprevT = l > 0 ? n->XT[l - 1] : n->X0T;
         const int splits = pick_splits(No, Ni, M);
-        float *out = splits > 1 ? n->part[l] : n->dW[l];
+        if ((L - 1 - l) % WGROUP == 0) part = n->part;
+        float *out = splits > 1 ? part : n->dW[l];
+        if (splits > 1) part += (size_t)splits * No * Ni;
         wgrads.push_back(npx::GemmF32{GT, XprevT, out, No, Ni, M, splits});
         finish.push_back(GradLayer{splits > 1 ? out : nullptr, n->dW[l], GT, n->db[l], splits, No, 0, (long long)No * Ni});
         if (l > 0) {
@@ -604,10 +617,11 @@ int npx_mlp_backward(npx_mlp *n, const float *x, const float *t, int M, float *l
     // The weight gradients together, after the chain that the others hang on.  One alone is a tile of
     // a few K blocks for each SM, whose epilogue nothing hides: four minibatches of 8,192 rows
     // (271 -> 4 x 512 -> 247) 1,025 -> 1,002 us.
-    RC(npx::gemm_group(wgrads.data(), L, n->err, n->stream));
-    for (int l = 0; l < L; l += GROUP) {
+    // (WGROUP layers' partials at a time: the next layers' products overwrite them)
+    for (int l = 0; l < L; l += WGROUP) {
         GradGroup group;
-        group.layers = std::min(GROUP, L - l);
+        group.layers = std::min(WGROUP, L - l);
+        RC(npx::gemm_group(wgrads.data() + l, group.layers, n->err, n->stream));
         int blocks = 0;
         for (int k = 0; k < group.layers; ++k) {
             GradLayer &g = group.l[k] = finish[l + k];

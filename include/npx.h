@@ -229,7 +229,15 @@ int npx_world_info_get(npx_world *w, npx_world_info *out);
 /* Launch shape of the step kernel: lanes per scene (4, 8, 16 or 32; a scene holds at most 64
  * points per lane), warps per block (1..16; shapes whose registers do not fit on an SM are refused
  * with NPX_ERANGE), resident blocks (0 = as many as fit), steps per kernel launch (chunk).  0 keeps
- * a value. */
+ * a value.  A shape within a few bytes per scene of an SM's shared memory runs with fewer warps per
+ * block than asked for (npx_world_info tells how many) until it fits; the results do not depend on
+ * the number.
+ * On flat ground without friction options or arenas, a world of more scenes than fit on the device
+ * at once may keep the posed points of the scenes in flight in device memory (16 bytes a point, at
+ * most 80 MB a size class), where that is faster; an explicit number of blocks keeps them in shared
+ * memory.  The device memory is allocated, after waiting for the world's stream, by the calls that lay
+ * the launches out: npx_world_finalize, this one, npx_world_autotune, npx_world_set_friction_model and
+ * npx_world_set_arenas.  Without it the points stay in shared memory. */
 int npx_world_configure(npx_world *w, int lanes_per_scene, int warps_per_block, int blocks,
                         int chunk_steps);
 /* Time the step kernel over the feasible launch shapes on a copy of the state (n_steps each)

@@ -107,12 +107,13 @@ struct WorldDev {
 
 struct LaunchCfg {
     int lps;      // lanes per scene: 4, 8, 16 or 32
-    int wpb;      // warps per block
+    int wpb;      // warps per block (of a launch: as many of those asked for as fit)
     int blocks;   // grid size
     int gp = 0;   // 1: the scenes' posed points in global memory (WorldDev::pscr), not in the slots
     int grid = 0; // 1: the caller asked for this grid size
     int slots = 0;  // 1: points stay in the slots (the autotuner timed that as the faster one)
     int gp_steps = 0;   // (gp) launches of fewer steps keep the points in the slots
+    int ask = 0;  // warps per block asked for; 0: wpb
 };
 
 int step_blocks_per_sm(const WorldDev &W, int lps, int wpb, int gp, cudaError_t *err);

@@ -326,11 +326,13 @@ npx::LaunchCfg clamp_cfg_for(npx_world *w, const npx::WorldDev &W, int count, np
     }
     cudaError_t e;
     c.gp = c.gp_steps = 0;
+    if (!c.ask) c.ask = c.wpb;
+    c.wpb = c.ask;
     if (!c.grid) c.blocks = 0;   // an automatic grid is sized anew
     int nb = npx::step_blocks_per_sm(W, c.lps, c.wpb, 0, &e);
     if (e != cudaSuccess) { *rc = fail(NPX_ECUDA, "occupancy query: %s", cudaGetErrorString(e)); return c; }
     // a shape that fits but for the tree numbers in the slots runs with fewer warps per block (the
-    // results do not depend on them)
+    // results do not depend on them) for as long as it does not fit
     if (nb < 1 && npx::step_fits_bare(W, c.lps, c.wpb))
         while (nb < 1 && c.wpb > 1 && e == cudaSuccess) nb = npx::step_blocks_per_sm(W, c.lps, --c.wpb, 0, &e);
     if (e != cudaSuccess) { *rc = fail(NPX_ECUDA, "occupancy query: %s", cudaGetErrorString(e)); return c; }
@@ -416,11 +418,11 @@ int scratch_fit(npx_world *w) {
     const bool fits = scratch_grow(w, n);
     int rc = NPX_OK;
     for (auto &c : w->classes) {
-        npx::LaunchCfg slots{c.cfg.lps, c.cfg.wpb, 0};
+        npx::LaunchCfg slots = c.cfg;
         slots.slots = 1;
         if (!fits) {
             c.poff = 0;
-            c.cfg = clamp_cfg_for(w, class_world(w, c), c.count, {c.cfg.lps, c.cfg.wpb, 0}, &rc);
+            c.cfg = clamp_cfg_for(w, class_world(w, c), c.count, c.cfg, &rc);
         }
         c.few = c.cfg.gp_steps ? clamp_cfg_for(w, class_world(w, c), c.count, slots, &rc) : c.cfg;
         if (rc) return rc;
@@ -1490,7 +1492,7 @@ int npx_world_configure(npx_world *w, int lps, int wpb, int blocks, int chunk) {
     }
     if (wpb) {
         if (wpb < 1 || wpb > 16) return fail(NPX_EINVAL, "warps per block must be 1..16");
-        c.wpb = wpb;
+        c.wpb = c.ask = wpb;
     }
     c.blocks = blocks > 0 ? blocks : (lps || wpb ? 0 : c.blocks);
     c.grid = blocks > 0 ? 1 : (lps || wpb ? 0 : c.grid);

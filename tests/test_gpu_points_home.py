@@ -78,3 +78,28 @@ def test_single_steps_are_not_slower_for_it(robots):
             best[i] = min(best[i], a.elapsed_time(e))
     assert best[0] < 1.25 * best[1], best
     _close(pair)
+
+
+def test_warps_asked_for_come_back_when_they_fit():
+    """A shape that fits but for the links' tree numbers runs with fewer warps per block; the number
+    asked for is kept for the shapes that follow."""
+    # 64 links and 876 points at 16 lanes: twelve slots leave no room for the tree numbers
+    pts = np.random.default_rng(0).uniform(-0.1, 0.1, (876, 3)).astype(np.float32)
+    n = np.full(64, 13)
+    n[:44] += 1
+    off = np.concatenate([[0], np.cumsum(n)])
+    links = [((0.2, 0.2, 0.2), (0, 0, 0), 1.0, k - 1, (0.0, 0.0, 0.0) if k else None,
+              (0.0, 0.0, 1.0) if k else None, -1) for k in range(64)]
+    b = scenes._assemble([(links, [pts[off[k]:off[k + 1]] for k in range(64)])] * 20, mu=np.full(20, 0.6),
+                         origin=np.tile([0, 0, 0.3], (20, 1)), quat=np.tile([1.0, 0, 0, 0], (20, 1)),
+                         vel=np.zeros((20, 3)), omega=np.tile([0.3, 0.2, 0.1], (20, 1)), act_params=None,
+                         name="edge", act_mode=scenes.ACT_HOLD)
+    w = World.from_batch(b, configure=dict(lanes_per_scene=16, warps_per_block=6))
+    assert w.info()["warps_per_block"] == 5
+    w.set_friction_model(3)
+    assert w.info()["warps_per_block"] == 5
+    w.configure(lanes_per_scene=32)
+    assert w.info()["warps_per_block"] == 6
+    w.step(3)
+    w.sync()
+    w.close()

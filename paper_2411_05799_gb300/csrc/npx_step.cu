@@ -597,7 +597,7 @@ __device__ __forceinline__ void scache_store(const WorldDev &W, int s, int np, c
 // Reads the posed shape of scene s (-1: no scene) from its cache entry into the slot: the offsets,
 // the mass properties and, when they were written with this many lanes per scene on every scene
 // of the warp, the tile boxes (else they are rebuilt from the offsets).  Returns rmax.
-template <int LPS, bool GP>
+template <int LPS>
 __device__ __forceinline__ float scache_load(const WorldDev &W, int s, int np, float4 *pts, float4 *tb, Shape &sh,
                                              int gl) {
     const float4 *e = W.scache + (size_t)(s < 0 ? 0 : s) * scache_stride(W.scache_mp, W.scache_mt, W.scache_ml);
@@ -609,10 +609,7 @@ __device__ __forceinline__ float scache_load(const WorldDev &W, int s, int np, f
     if (s >= 0) { m0 = m[0]; m1 = m[1]; m2 = m[2]; m3 = m[3]; m4 = m[4]; }
     const bool tb_ok = __all_sync(FULL_MASK, __float_as_int(m4.y) == LPS);
 #pragma unroll 4
-    for (int i = gl; i < np; i += LPS) {
-        if constexpr (GP) pts[i] = e[i];
-        else cp_async16(pts + i, e + i);
-    }
+    for (int i = gl; i < np; i += LPS) cp_async16(pts + i, e + i);
     if (tb_ok)
         for (int i = gl; i < 2 * nt; i += LPS) cp_async16(tb + i, e + W.scache_mp + i);
     cp_async_wait_all();
@@ -1289,13 +1286,18 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
     Shape sh;
     float rmax;
     // the posed shape of the current joint angles: read from the posed-shape cache when the
-    // launch says every entry is current, else rebuilt (and written to the cache when there is one)
-    if (!ARENA && W.scache_mode == 2) {
-        rmax = scache_load<LPS, GP>(W, valid ? s : -1, np, pts, tb, sh, gl);
-    } else {
+    // launch says every entry is current, else rebuilt (and written to the cache when there is one);
+    // the launches with a cache are the surrogate's, whose points are in the slots
+    constexpr bool CACHE = !ARENA && !GP;
+    bool cached = false;
+    if constexpr (CACHE) {
+        cached = W.scache_mode == 2;
+        if (cached) rmax = scache_load<LPS>(W, valid ? s : -1, np, pts, tb, sh, gl);
+    }
+    if (!cached) {
         shape_update<LPS, GP>(W, valid ? s : 0, p0, np, l0, nl, th, fr, pts, gl, sh);
         rmax = tile_bounds<LPS>(pts, np, tb, gl);
-        if (!ARENA && W.scache_mode != 0 && valid) scache_store<LPS>(W, s, np, pts, tb, sh, rmax, fr, l0, nl, gl);
+        if (CACHE && W.scache_mode != 0 && valid) scache_store<LPS>(W, s, np, pts, tb, sh, rmax, fr, l0, nl, gl);
     }
     // (arenas) body-frame box of the posed points
     float bbc[3] = {0.f, 0.f, 0.f}, bbh[3] = {0.f, 0.f, 0.f};
@@ -1404,7 +1406,7 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
             __syncwarp();
             shape_update<LPS, GP>(W, valid ? s : 0, p0, np, l0, nl, th, fr, pts, gl, sh);
             rmax = tile_bounds<LPS>(pts, np, tb, gl);
-            if (!ARENA && W.scache_mode != 0 && valid) scache_store<LPS>(W, s, np, pts, tb, sh, rmax, fr, l0, nl, gl);
+            if (CACHE && W.scache_mode != 0 && valid) scache_store<LPS>(W, s, np, pts, tb, sh, rmax, fr, l0, nl, gl);
             shr = sh;
             if (ARENA) {
                 robot_box<LPS>(tb, ntiles, gl, bbc, bbh);
@@ -2856,7 +2858,7 @@ int step_blocks_per_sm(const WorldDev &W, int lps, int wpb, int gp, cudaError_t 
 
 cudaError_t launch_step(const WorldDev &W, const LaunchCfg &cfg, int n_steps, cudaStream_t st) {
     void *fn = pick_step(W, cfg.lps, cfg.gp);
-    if (!fn || cfg.wpb < 1 || cfg.wpb > 16 || cfg.blocks < 1 || (cfg.gp && !W.pscr)) return cudaErrorInvalidValue;
+    if (!fn || cfg.wpb < 1 || cfg.wpb > 16 || cfg.blocks < 1 || (cfg.gp && (!W.pscr || W.scache_mode))) return cudaErrorInvalidValue;
     // the kernel's shared-memory limit was raised by step_blocks_per_sm for this shape
     const size_t smem = step_smem_bytes(W, cfg.lps, cfg.wpb, cfg.gp);
     cudaError_t e = cudaMemsetAsync(W.queue, 0, sizeof(unsigned int), st);

@@ -1278,7 +1278,10 @@ __device__ void run_scene(const WorldDev &W, int s, int gl, float4 *pts, float *
     for (int j = gl; j < nj; j += LPS) th[j] = W.theta[j0 + j];
     uint64_t kprev = 0;
     if (!W.reseed) {
-#pragma unroll 8
+        // (loads in flight; a lane of 32 has no 16 flags of a hexapod's 352: one step of 16,384 hexapods,
+        // 8 lanes, 67.5 us with 8 and 65.8 with 16; 80 steps of one, 32 lanes, 132.5 and 134.3)
+        constexpr int AHEAD = LPS <= 16 ? 16 : 8;
+#pragma unroll AHEAD
         for (int k = 0, i = gl; i < np; ++k, i += LPS)
             if (W.kappa[p0 + i]) kprev |= 1ull << k;
     }

@@ -103,3 +103,50 @@ def test_warps_asked_for_come_back_when_they_fit():
     w.step(3)
     w.sync()
     w.close()
+
+
+def _same(pair):
+    r, q = (w.read() for w in pair)
+    for k in KEYS:
+        np.testing.assert_array_equal(r[k], q[k], err_msg=k)
+    np.testing.assert_array_equal(pair[0].contacts(), pair[1].contacts())
+
+
+@pytest.mark.parametrize("lanes, warps, robots, least, most", [
+    (4, 2, 14000, 129, 256), (8, 3, 11000, 300, 512), (16, 2, 2500, 513, 1024), (32, 2, 1500, 1025, 2048),
+    (32, 3, 1501, 1, 2048)])
+def test_every_build_at_the_sizes_that_take_it(lanes, warps, robots, least, most):
+    """The points are in global memory (more blocks run than the slots have room for), and the results
+    are the slots' bit for bit, from the smallest to the largest scene of each build."""
+    b = scenes.ragged_bodies([least + (97 * i) % (most + 1 - least) for i in range(robots)], seed_key=lanes)
+    pair = _pair(b, lanes, warps)
+    assert _global(pair)
+    for w in pair:
+        for n in (170, 17, 160):
+            w.step(n)
+    _same(pair)
+    _close(pair)
+
+
+def test_changes_of_model_and_shape_between_steps():
+    """A world that leaves global memory for the friction options and for arenas and comes back, and
+    whose scratch grows under captured graphs: bit for bit what an explicit grid gives throughout."""
+    pair = _pair(scenes.arena_batch(2250, 4, seed_key=6), 8, 7)
+    assert _global(pair)
+
+    def each(f, home):
+        for i, w in enumerate(pair):
+            f(w, {"blocks": 100000} if i else {})
+            w.step(45)
+        assert _global(pair) == home
+        _same(pair)
+
+    each(lambda w, grid: None, True)
+    each(lambda w, grid: w.configure(lanes_per_scene=8, warps_per_block=2, **grid), True)    # the scratch grows
+    each(lambda w, grid: w.set_friction_model(3), False)
+    each(lambda w, grid: w.set_friction_model(0), True)
+    each(lambda w, grid: w.set_arenas(4, 0.01), False)
+    each(lambda w, grid: w.set_arenas(1), True)
+    each(lambda w, grid: w.configure(lanes_per_scene=8, warps_per_block=1, **grid), True)
+    each(lambda w, grid: w.use_graphs(False), True)
+    _close(pair)

@@ -66,7 +66,7 @@ int npx_gemm_warp_wait_selftest(int *split, int *complete, void *stream);
 
 /* --- the surrogate network --------------------------------------------------------------
  * y = W_L gelu(... gelu(W_1 x + b_1) ...) + b_L with n_hidden_layers GELU layers of width
- * n_hidden (exact GELU, z Phi(z)), trained on the mean over the batch of the squared error summed
+ * n_hidden (GELU in its tanh form), trained on the mean over the batch of the squared error summed
  * over outputs, with Adam.  Master weights, gradients and Adam moments are FP32; the GEMMs read
  * BF16 copies of the weights and BF16 activations and accumulate in FP32.  Inputs are zero-padded
  * to a multiple of 128 features and outputs to a multiple of 128 (the padding never reaches the

@@ -147,8 +147,6 @@ __device__ __forceinline__ void epilogue16(const npx_gemm_epilogue &ep, float (&
     }
 }
 
-// STORE = 2: the FP32 row-major output (outf) leaves through per-warp shared-memory boxes and TMA
-// stores (tout); STORE = 0: every output is stored directly.
 // G products in one launch: their tiles (and split-K ranges) form one list, walked by the persistent
 // blocks, so that a product's epilogues run under the next one's copies and MMAs.
 template <int G>
@@ -178,6 +176,8 @@ __device__ __forceinline__ Tile tile_at(const Products<G> &P, int t) {
     return r;
 }
 
+// STORE = 2: the FP32 row-major output (outf) leaves through per-warp shared-memory boxes and TMA
+// stores (P.out), STORE = 1: the BF16 one (out) does; STORE = 0: every output is stored directly.
 template <int BN, int STORE, int G>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_tn_kernel(const __grid_constant__ Products<G> P, npx_gemm_epilogue ep, int *err) {

@@ -240,8 +240,8 @@ namespace npx {
 // when the kernel before, which itself waited for its own, has ended and its writes are visible),
 // and early_next where its successor may start.  None takes a pointer as const __restrict__ or loads
 // by __ldg: that promises memory which stays as it is for as long as the kernel lives, and its life
-// begins while the kernel ahead still writes.  A training step is 18 launches of 3 to 15 us: four
-// minibatches of 8,192 rows (271 -> 4 x 512 -> 247) 1,178 -> 1,025 us.
+// begins while the kernel ahead still writes.  A training step is 15 kernels of 3 to 27 us (18 when
+// this came: four minibatches of 8,192 rows, 271 -> 4 x 512 -> 247, 1,178 -> 1,025 us).
 __device__ __forceinline__ void early_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void early_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(256) loss_grad_kernel(const float *Y, const fl
 // of the layer's transposed output gradient GT [rows x M] (read from the transpose so that every load
 // is a full line).  Bound by launches: layer by layer these were ten launches of 4 to 6 us each,
 // 49 us of a 357 us minibatch of 8,192 rows (271 -> 4 x 512 -> 247); with Adam's ten below as one, a
-// minibatch took 294 us.
+// minibatch took 294 us (235 now).
 constexpr int WGROUP = npx::GEMM_GROUP;   // layers whose weight gradients are formed together
 struct GradLayer {
     const float *part;      // [splits][n], or NULL: the gradient is written already
@@ -228,8 +228,8 @@ inline unsigned blocks_for(long long n, int t = 256) { return (unsigned)((n + t 
 // added in a fixed order (the blocks' sums over distributed shared memory, so there is no
 // workspace and no atomic): every column's sum repeats bit for bit.
 // Bound by the FP64 pipe (an add and a fused multiply-add per element, two lanes a clock and SM on
-// this part), so the work has to reach every SM: 65,536 x 271 took 1.80 ms on the nine blocks of
-// one 32-column block each, 0.17 ms on 272.
+// this part), so the work has to reach every SM: 65,536 x 271 took 590 us on nine blocks of 32 columns
+// each, 102 us on 272 (the first pass on new rows 1.80 ms and 0.17 ms).
 constexpr int MOM_CTAS = 8, MOM_THREADS = 256;
 
 template <int CW>

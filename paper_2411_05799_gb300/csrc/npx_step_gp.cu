@@ -7,8 +7,8 @@
 // Flat ground with the points in global memory: a slot is a third of its size (hexapods 2.6 of 8.2
 // KB), so registers (16 warps per SM) and not shared memory (7 at 8 lanes) bound the scenes in
 // flight, and the few points a step touches are L1 hits.  Taken by chunked stepping where not every
-// scene fits on the device at once (npx_world.cpp): evolution of 16,000 hexapods, 400 steps: 3.58 -> 2.75 ms.
-// Launches of a few steps, and worlds whose joints move at most steps, keep them in the slots.
+// scene fits on the device at once: evolution of 16,000 hexapods, 400 steps: 3.58 -> 2.53 ms.  The rule
+// in npx_world.cpp says which worlds, and which launches of few steps, keep them in the slots.
 template <int LPS>
 __global__ void __launch_bounds__(512) step_kernel_gp(const __grid_constant__ WorldDev W, int n_steps, int sbytes,
                                                       const __grid_constant__ CUtensorMap tmap) {
